@@ -26,6 +26,7 @@
 
 #include <type_traits>
 
+#include "lbm_fixed.cuh"
 #include "lbm_fp64emu.cuh"
 
 namespace olbm {
@@ -118,8 +119,13 @@ struct Geometry {
   long long plane;  // elements between planes
 };
 
-// Per-run coefficients, computed once on the host in FP64 and rounded to T.
-template <typename T> struct Coef {
+// Per-run coefficients, computed once on the host in FP64 and rounded to T; FP64
+// also carries those of the fixed-point collision.
+template <typename T> struct FixedPart {};
+template <> struct FixedPart<double> {
+  fx::Coefs fixed;
+};
+template <typename T> struct Coef : FixedPart<T> {
   T theta;        // theta
   T one_m_theta;  // 1 - theta            (P(0) at u = 0)
   T half_theta;   // theta / 2            (P(+-1) at u = 0)
@@ -163,6 +169,7 @@ template <typename T> __host__ Coef<T> make_coef(double theta, double tau, doubl
   c.rwp = (T)(rho_ref * 0.5 * theta);
   c.nrw0 = (T)(-rho_ref * (1.0 - theta));
   c.nrwp = (T)(-rho_ref * 0.5 * theta);
+  if constexpr (std::is_same<T, double>::value) c.fixed = fx::make_coefs(theta, tau);
   return c;
 }
 
@@ -485,16 +492,16 @@ __device__ __forceinline__ void collide_form(T (&f)[9], const Coef<T>& c, Sink&&
 }
 
 // FP64 values whose products run on the integer pipes (emu::mul64, bit-identical
-// to the FP64 instruction); sums and FMAs stay on the FP64 pipe. The FP64
-// collision runs on this type, so the FP64 pipe, which bounds the FP64 form on
-// GB300, carries only the sums and FMAs, while the products overlap with them on
-// the otherwise idle integer pipes (complete model at 4096^2, diagnostics every
-// step: 4.78 -> 6.33 GLUPS). The products leave out their fallback (a product
-// outside the fast path is a quiet NaN), and collide() checks the node's nine
-// results once instead: a branch per product measured 6 % slower. Sums on the
-// integer pipes as well (emu::add64) measured slower wherever they were put: the
-// moments, which head the collision's dependency chain, 4.9; the corrections,
-// the factors P or C, or the diagnostics sums, 5.2 to 5.6 (against 5.76).
+// to the FP64 instruction); sums and FMAs stay on the FP64 pipe. The floating-point
+// FP64 collision (nodes outside the fixed-point range, see collide_fixed) and the
+// adjoint step run on these types, so the FP64 pipe, which bounds them on GB300,
+// carries only the sums and FMAs, while the products overlap with them on the
+// otherwise idle integer pipes (complete model at 4096^2, every node on this path,
+// diagnostics every step: 4.78 -> 6.33 GLUPS). The products leave out their fallback
+// (a product outside the fast path is a quiet NaN), and collide() checks the node's
+// nine results once instead: a branch per product measured 6 % slower. Sums on the
+// integer pipes as well (emu::add64, about 60 instructions each) measured slower
+// wherever they were put.
 #ifndef OLBM_F64_EMU_MUL
 #define OLBM_F64_EMU_MUL 1
 #endif
@@ -560,8 +567,8 @@ struct KeepInputs {
 // with zero operands on the fast path (zeros come in regions: a flow at rest, a
 // velocity component that vanishes everywhere), 2 the FP64 products.
 template <int MODEL, bool SHIFT, typename T, typename Sink, typename Refetch = KeepInputs>
-__device__ __forceinline__ void collide(T (&f)[9], const Coef<T>& c, Sink&& sink, Refetch&& refetch = Refetch(),
-                                        int* mode = nullptr) {
+__device__ __forceinline__ void collide(T (&f)[9], const Coef<T>& c, Sink&& sink,
+                                              Refetch&& refetch = Refetch(), int* mode = nullptr) {
   if constexpr (std::is_same<T, double>::value && OLBM_F64_EMU_MUL) {
     constexpr bool kKeep = std::is_same<std::decay_t<Refetch>, KeepInputs>::value;
     auto to_double = [&](const auto& m) {
@@ -618,6 +625,52 @@ __device__ __forceinline__ void collide(T (&f)[9], const Coef<T>& c, Sink&& sink
   } else {
     collide_form<MODEL, SHIFT, T>(f, c, sink);
   }
+}
+
+// What the fixed-point collision hands to the diagnostics.
+struct FixedMoments {
+  long long rho, jx, jy, ke2;  // 60 fraction bits; ke2 = j.u, twice the kinetic energy
+};
+
+// Collision of one FP64 node in fixed point (lbm_fixed.cuh); false for a node outside its
+// range, for which nothing is stored: that is a property of the node alone. next(f) is called
+// as soon as f is free and may load the next node's populations into it; sink receives the
+// node's FixedMoments and store(i, v) each post-collision population.
+template <int MODEL, typename Sink, typename Next, typename Store>
+__device__ __forceinline__ bool collide_fixed(double (&f)[9], const Coef<double>& c, Sink&& sink, Next&& next,
+                                              Store&& store) {
+  fx::Fx<60> a[9], o[9];
+  // sign and magnitude of all nine at once: +0 <= f_i < 1 is the common case
+  unsigned top = 0;
+#pragma unroll
+  for (int i = 0; i < 9; ++i) top = max(top, (unsigned)__double2hiint(f[i]));
+  bool ok = top < 0x3FF00000u;
+  if (__all_sync(__activemask(), ok)) {
+#pragma unroll
+    for (int i = 0; i < 9; ++i) a[i] = fx::nonnegative(f[i]);
+  } else {
+    ok = true;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+      a[i] = fx::any_sign(f[i]);
+      ok = ok && ((unsigned)__double2hiint(f[i]) & 0x7FFFFFFFu) < 0x3FF00000u;
+    }
+  }
+  next(f);
+  const fx::Moments m = fx::moments(a);
+  ok = ok && fx::moments_in_range(m.rho, m.jx, m.jy);
+  if (!__any_sync(__activemask(), ok)) return false;
+  fx::Fx<60> ke2;
+  ok = ok && fx::collide<MODEL>(m, a, c.fixed, o, ke2);
+  if (ok) {
+    sink(FixedMoments{m.rho.v, m.jx.v, m.jy.v, ke2.v});
+    store(0, fx::to_double(o[0]));
+#pragma unroll
+    for (int i = 1; i < 5; ++i) store(i, fx::to_double(fx::Fx<61>{o[i].v}));
+#pragma unroll
+    for (int i = 5; i < 9; ++i) store(i, fx::to_double(fx::Fx<62>{o[i].v}));
+  }
+  return ok;
 }
 
 // Per-axis factor of the guided equilibrium (Eq. 10) in FP64, for velocity

@@ -164,6 +164,52 @@ template <typename CT> struct DiagAcc {
     }
   }
 };
+// FP64: nodes of the fixed-point path add into 96-bit integer sums (exact; four
+// 32-bit instructions a sum, where an FP64 addition holds its pipe for 64 cycles),
+// the others into FP64 ones.
+struct Sum96 {
+  unsigned lo = 0, mid = 0;
+  int hi = 0;
+  __device__ __forceinline__ void add(long long v) {
+    asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.s32 %2, %2, %5;"
+        : "+r"(lo), "+r"(mid), "+r"(hi)
+        : "r"((unsigned)v), "r"((unsigned)(v >> 32)), "r"((int)(v >> 63)));
+  }
+  // The sum in units of 2^-60, the low 64 bits taken as a signed number.
+  __device__ __forceinline__ double value() const {
+    const long long low = (long long)(((unsigned long long)mid << 32) | lo);
+    return fma((double)(hi + (int)(mid >> 31)), 16.0, (double)low * 0x1p-60);
+  }
+};
+template <> struct DiagAcc<double> {
+  double v[4];
+  int bad;
+  Sum96 s[4];
+  __device__ DiagAcc() : bad(0) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] = 0.0;
+  }
+  __device__ __forceinline__ void add(const NodeMoments<double>& m) {
+    if (finite_lead(m.m0)) {
+      v[0] += m.m0;
+      v[1] += m.jx;
+      v[2] += m.jy;
+      v[3] = fma(m.jx, m.ux, fma(m.jy, m.uy, v[3]));
+    } else {
+      ++bad;
+    }
+  }
+  __device__ __forceinline__ void add(const FixedMoments& m) {
+    s[0].add(m.rho);
+    s[1].add(m.jx);
+    s[2].add(m.jy);
+    s[3].add(m.ke2);
+  }
+  __device__ __forceinline__ void merge() {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] += s[k].value();
+  }
+};
 // Packed pairs accumulate into four FP32 scalars: both nodes of a pair go into
 // the same sums, which holds four registers fewer through the collision than
 // packed sums would (measured on the FP16 form at 4096^2 with diagnostics every
@@ -195,6 +241,7 @@ template <> struct DiagAcc<f32x2> {
 
 // Reduce a thread's accumulator over the block into out5 (thread 0 writes).
 template <typename CT> __device__ __forceinline__ void block_diag_acc(DiagAcc<CT>& a, double* out5) {
+  if constexpr (std::is_same<CT, double>::value) a.merge();
   a.v[3] = scaled(a.v[3], 0.5f);  // kinetic energy
   if constexpr (std::is_same<CT, f32x2>::value) {
     block_diag<float>(a.v, a.bad, out5);
@@ -256,6 +303,34 @@ template <int MODEL, int PREC, bool DIAG, bool PAIRS, bool CG = false> struct Co
     }
   }
 
+  // FP64, floating point: the rows r of the column with bit r of `left` set. Out of line:
+  // the rows that the fixed-point collision leaves out are rare, and its registers would
+  // burden the loop that handles the others.
+  __device__ static __noinline__ void run_float(const S* __restrict__ src, S* __restrict__ dst, const Geometry& g,
+                                                const Coef<CT>& c, int x, int xm, int xp, int y0, int dy, int rows,
+                                                unsigned long long left, DiagAcc<CT>& acc) {
+    int mode = 0;  // which products this warp's nodes take (see collide)
+    for (int r = 0, y = y0; r < rows && y < g.ny; ++r, y += dy) {
+      const bool mine = (left >> r) & 1;
+      const unsigned warp = __activemask();
+      if (!__any_sync(warp, mine)) continue;
+      if (mine) {
+        CT f[9];
+        pull(src, g, x, xm, xp, y, f);
+        collide<MODEL, false, CT>(
+            f, c,
+            [&](const NodeMoments<CT>& m) {
+              if constexpr (DIAG) acc.add(m);
+            },
+            [&](CT (&h)[9]) { pull(src, g, x, xm, xp, y, h); }, &mode);
+        S* q = dst + (long long)y * g.pitch + x;
+#pragma unroll
+        for (int i = 0; i < 9; ++i) st_t(q + i * g.plane, f[i]);
+      }
+      __syncwarp(warp);
+    }
+  }
+
   __device__ static __forceinline__ void run(const S* __restrict__ src, S* __restrict__ dst, const Geometry& g,
                                              const Coef<CT>& c, int x, int y0, int dy, int rows,
                                              DiagAcc<CT>& acc) {
@@ -293,19 +368,47 @@ template <int MODEL, int PREC, bool DIAG, bool PAIRS, bool CG = false> struct Co
       }
       return;
     }
+    auto sink = [&](const auto& m) {
+      if constexpr (DIAG) acc.add(m);
+    };
+    if constexpr (PREC == 0) {
+      // FP64: the rows in fixed point, the next row's loads going into f once its row is
+      // converted; then the rows it left out (bit r of `left`; rows <= 64) in floating point.
+      unsigned long long left = ~0ull;
+      if (c.fixed.on) {
+        left = 0;
+        double f[9];
+        int y = y0;
+        if (y < g.ny) pull(src, g, x, xm, xp, y, f);
+        for (int r = 0; r < rows && y < g.ny; ++r, y += dy) {
+          double* q = dst + (long long)y * g.pitch + x;
+          const bool done = collide_fixed<MODEL>(
+              f, c, sink,
+              [&](double (&h)[9]) {
+                if ((r + 1 < rows) && (y + dy < g.ny)) pull(src, g, x, xm, xp, y + dy, h);
+              },
+              [&](int i, double v) { q[i * g.plane] = v; });
+          left |= done ? 0ull : 1ull << r;
+        }
+      }
+      if (__any_sync(__activemask(), left != 0)) {
+        DiagAcc<CT> rest;  // (acc itself stays in registers: its address goes nowhere)
+        run_float(src, dst, g, c, x, xm, xp, y0, dy, rows, left, rest);
+        if constexpr (DIAG) {
+#pragma unroll
+          for (int k = 0; k < 4; ++k) acc.v[k] += rest.v[k];
+          acc.bad += rest.bad;
+        }
+      }
+      return;
+    }
     CT f[9], fn[9];
     int y = y0;
-    int mode = 0;  // FP64: which products this warp's nodes take (see collide)
     if (y < g.ny) pull(src, g, x, xm, xp, y, f);
     for (int r = 0; r < rows && y < g.ny; ++r, y += dy) {
       const bool more = (r + 1 < rows) && (y + dy < g.ny);
       if (more) pull(src, g, x, xm, xp, y + dy, fn);
-      collide<MODEL, Form<PREC>::kShift, CT>(
-          f, c,
-          [&](const NodeMoments<CT>& m) {
-            if constexpr (DIAG) acc.add(m);
-          },
-          [&](CT (&r)[9]) { pull(src, g, x, xm, xp, y, r); }, &mode);
+      collide<MODEL, Form<PREC>::kShift, CT>(f, c, sink);
       S* q = dst + (long long)y * g.pitch + x;
       if constexpr (PAIRS) {
 #pragma unroll
@@ -364,14 +467,15 @@ __global__ void __maxnreg__(OLBM_DF_MAXNREG) step_kernel_df(const double* __rest
   step_body<MODEL, 3, DIAG, PAIRS>(src, dst, g, c, partials, rows);
 }
 
-// The FP64 form is bound by the FP64 pipe. With its products on the integer
-// pipes it is capped at 128 registers a thread (four blocks of 128 threads an
-// SM, a few bytes spilled): the cap raised the 4096^2 rate from 5.57 to 5.77
-// GLUPS when it was set. With every product on the FP64 pipe the rate measured
-// the same for caps from 72 (seven blocks, spilling) to 128 registers
-// (4751-4762 MLUPS). Launched with at most 512 threads.
+// The FP64 form collides in 64-bit fixed point on the integer pipes (lbm_fixed.cuh),
+// which bound it: ALU, FMA-heavy (the wide products) and issue are each about 60 %
+// busy. Complete model at 4096^2, diagnostics every step / off: 31.8 / 34.5 GLUPS
+// (6.33 / 6.8 with the collision on the FP64 pipe, its products on the integer pipes).
+// Capped at 96 registers a thread, five blocks of 128 threads an SM, without spills in
+// the row loop (128: 31.6 / 33.2, 88: 31.7 / 34.0, 80: 32.1 / 34.1, 72: 31.6 / 33.7).
+// Launched with at most 512 threads.
 #ifndef OLBM_F64_MAXNREG
-#define OLBM_F64_MAXNREG 128
+#define OLBM_F64_MAXNREG 96
 #endif
 template <int MODEL, bool DIAG>
 __global__ void __maxnreg__(OLBM_F64_MAXNREG) step_kernel_f64(const double* __restrict__ src, double* __restrict__ dst, Geometry g,

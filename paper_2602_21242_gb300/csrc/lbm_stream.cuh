@@ -370,15 +370,20 @@ template <int PREC, int NC, int STAGES> struct Pipeline {
       __syncwarp();
       if (lane == 0) mbar_arrive(&empty[s]);
       if (active) {
-        collide<MODEL, false, double>(
-            f, c,
-            [&](const NodeMoments<double>& m) {
-              if constexpr (DIAG) acc.add(m);
-            },
-            KeepInputs(), &mode);
         double* q = dst + (long long)(y0 + r0 + j) * g.pitch + x0 + xl;
+        auto sink = [&](const auto& m) {
+          if constexpr (DIAG) acc.add(m);
+        };
+        auto store = [&](int i, double v) { q[i * g.plane] = v; };
+        double h[9];
 #pragma unroll
-        for (int i = 0; i < 9; ++i) q[i * g.plane] = f[i];
+        for (int i = 0; i < 9; ++i) h[i] = f[i];
+        const bool left = !c.fixed.on || !collide_fixed<MODEL>(h, c, sink, [](double (&)[9]) {}, store);
+        if (__any_sync(__activemask(), left) && left) {
+          collide<MODEL, false, double>(f, c, sink, KeepInputs(), &mode);
+#pragma unroll
+          for (int i = 0; i < 9; ++i) store(i, f[i]);
+        }
       }
     }
     return true;
