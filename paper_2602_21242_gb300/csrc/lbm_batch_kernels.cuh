@@ -31,15 +31,24 @@ __device__ __forceinline__ void update_tile(const Desc<typename Form<PREC>::T>& 
     if (d.pairs) {
       using Col = Column<MODEL, PREC, DIAG, true, CG>;
       DiagAcc<f32x2> acc;
-      Col::run(src, dst, d.g, broadcast(d.c), x0 + 2 * threadIdx.x, y, dy, rows, acc);
+      FixedDiagAcc none;
+      Col::template run<false>(src, dst, d.g, broadcast(d.c), x0 + 2 * threadIdx.x, y, dy, rows, acc, none);
       if constexpr (DIAG) block_diag_acc(acc, out5);
       return;
     }
   }
   using Col = Column<MODEL, PREC, DIAG, false, CG>;
   DiagAcc<typename Col::CT> acc;
-  Col::run(src, dst, d.g, d.c, x0 + threadIdx.x, y, dy, rows, acc);
-  if constexpr (DIAG) block_diag_acc(acc, out5);
+  FixedDiagAcc facc;
+  if constexpr (PREC == 0) {
+    if (d.c.fixed.on)
+      Col::template run<true>(src, dst, d.g, d.c, x0 + threadIdx.x, y, dy, rows, acc, facc);
+    else
+      Col::template run<false>(src, dst, d.g, d.c, x0 + threadIdx.x, y, dy, rows, acc, facc);
+  } else {
+    Col::template run<false>(src, dst, d.g, d.c, x0 + threadIdx.x, y, dy, rows, acc, facc);
+  }
+  if constexpr (DIAG) block_diag_acc(acc, out5, &facc);
 }
 
 // One time step of every domain: block b updates tile b.

@@ -119,10 +119,12 @@ struct Geometry {
   long long plane;  // elements between planes
 };
 
-// Per-run coefficients, computed once on the host in FP64 and rounded to T; FP64
-// also carries those of the fixed-point collision.
-template <typename T> struct FixedPart {};
-template <> struct FixedPart<double> {
+// Per-run coefficients, computed once on the host in FP64 and rounded to T; the forms
+// with FP64 storage also carry those of the fixed-point collision.
+struct df64;  // double-word FP32 (lbm_df64.cuh)
+template <typename T> constexpr bool kHasFixed = std::is_same<T, double>::value || std::is_same<T, df64>::value;
+template <typename T, bool = kHasFixed<T>> struct FixedPart {};
+template <typename T> struct FixedPart<T, true> {
   fx::Coefs fixed;
 };
 template <typename T> struct Coef : FixedPart<T> {
@@ -169,7 +171,7 @@ template <typename T> __host__ Coef<T> make_coef(double theta, double tau, doubl
   c.rwp = (T)(rho_ref * 0.5 * theta);
   c.nrw0 = (T)(-rho_ref * (1.0 - theta));
   c.nrwp = (T)(-rho_ref * 0.5 * theta);
-  if constexpr (std::is_same<T, double>::value) c.fixed = fx::make_coefs(theta, tau);
+  if constexpr (kHasFixed<T>) c.fixed = fx::make_coefs(theta, tau);
   return c;
 }
 
@@ -637,7 +639,7 @@ struct FixedMoments {
 // as soon as f is free and may load the next node's populations into it; sink receives the
 // node's FixedMoments and store(i, v) each post-collision population.
 template <int MODEL, typename Sink, typename Next, typename Store>
-__device__ __forceinline__ bool collide_fixed(double (&f)[9], const Coef<double>& c, Sink&& sink, Next&& next,
+__device__ __forceinline__ bool collide_fixed(double (&f)[9], const fx::Coefs& c, Sink&& sink, Next&& next,
                                               Store&& store) {
   fx::Fx<60> a[9], o[9];
   // sign and magnitude of all nine at once: +0 <= f_i < 1 is the common case
@@ -661,7 +663,7 @@ __device__ __forceinline__ bool collide_fixed(double (&f)[9], const Coef<double>
   ok = ok && fx::moments_in_range(m.rho, m.jx, m.jy);
   if (!__any_sync(__activemask(), ok)) return false;
   fx::Fx<60> ke2;
-  ok = ok && fx::collide<MODEL>(m, a, c.fixed, o, ke2);
+  ok = ok && fx::collide<MODEL>(m, a, c, o, ke2);
   if (ok) {
     sink(FixedMoments{m.rho.v, m.jx.v, m.jy.v, ke2.v});
     store(0, fx::to_double(o[0]));

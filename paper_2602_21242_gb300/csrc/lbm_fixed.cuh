@@ -39,7 +39,7 @@
 // Range. A node takes this path when its populations are below 1 in magnitude, its
 // density lies in [1/2, 4), its velocity components are below 1/2, its normal and
 // shear non-equilibrium stresses below 1/2 and |A1| < 1, theta lies in
-// [0.21, 0.57] and tau is at most 1e9; every other node (a blown-up state, another unit of density) goes to
+// [0.21, 0.65] and tau is at most 1e9; every other node (a blown-up state, another unit of density) goes to
 // the floating-point collision. The choice depends on the node alone, so results do
 // not depend on which nodes share a warp. The ranges below are those that the
 // formats written as Fx<fraction bits> need; each value stays below 2^63 in its format.
@@ -147,7 +147,7 @@ struct Coefs {
   FxOp<60> q2;         // 1 / (4 theta^2)
   FxOp<60> inv_theta;  // 1 / theta
   FxOp<61> e2;         // (1 - theta) / (2 theta) (polynomial equilibrium)
-  Fx<63> theta, h, t, c3;
+  Fx<62> theta, h, t, c3;
   Fx<60> v0;           // (1 - theta) / theta
   int on;              // theta in the range of the formats
 };
@@ -161,7 +161,7 @@ template <int F> inline Fx<F> fx_of(long double x) {
 inline Coefs make_coefs(double theta, double tau) {
   Coefs c;
   memset(&c, 0, sizeof c);
-  c.on = theta >= 0.21 && theta <= 0.57 && tau <= 1e9 ? 1 : 0;  // omega' < 1 with 63 fraction bits
+  c.on = theta >= 0.21 && theta <= 0.65 && tau <= 1e9 ? 1 : 0;  // omega' < 1 with 63 fraction bits
   if (!c.on) return c;
   const long double th = theta, omp = 1.0L - 1.0L / tau;
   c.k1 = op(fx_of<60>(omp / (4.0L * th * th)));
@@ -170,10 +170,10 @@ inline Coefs make_coefs(double theta, double tau) {
   c.q2 = op(fx_of<60>(1.0L / (4.0L * th * th)));
   c.inv_theta = op(fx_of<60>(1.0L / th));
   c.e2 = op(fx_of<61>((1.0L - th) / (2.0L * th)));
-  c.theta = fx_of<63>(th);
-  c.h = fx_of<63>(th * (1.0L - th));
-  c.t = fx_of<63>(th * (1.0L - 3.0L * th));
-  c.c3 = fx_of<63>(1.0L - 3.0L * th);
+  c.theta = fx_of<62>(th);
+  c.h = fx_of<62>(th * (1.0L - th));
+  c.t = fx_of<62>(th * (1.0L - 3.0L * th));
+  c.c3 = fx_of<62>(1.0L - 3.0L * th);
   c.v0 = fx_of<60>((1.0L - th) / th);
   return c;
 }
@@ -304,7 +304,7 @@ OLBM_EMU_HD bool collide(const Moments& m, const Fx<60> (&f)[9], const Coefs& c,
   if constexpr (MODEL == 0) {
     M20 = rsx, M02 = rsy, M11 = jxuy;
     M21 = op(rsx) * uy, M12 = op(rsy) * ux;
-    M22 = op(to<61>(rsx)) * op(c.theta + to<63>(uy2));
+    M22 = to<60>(op(to<61>(rsx)) * op(c.theta + to<62>(uy2)));
   } else if constexpr (MODEL == 5) {
     // polynomial equilibrium: rho (theta + u_a^2 (1 - theta)/(2 theta)), rho theta u, and
     // rho (theta^2 + |u|^2 (1 - theta)/2)
@@ -317,23 +317,22 @@ OLBM_EMU_HD bool collide(const Moments& m, const Fx<60> (&f)[9], const Coefs& c,
     ok = within(E.v, 1 << 27) & within(N.v, 1 << 27);
     const Fx<60> A1 = op(to<64>(E)) * c.k1;  // |k1| <= 5.7, |E| < 1/2
     ok = ok & within(A1.v, 1 << 28);
-    const FxOp<61> A1o = op(to<61>(A1));
-    const Fx<63> ux2h = to<63>(ux2), uy2h = to<63>(uy2);
-    const Fx<63> X = to<63>(square(op(ux2))) - ux2h, Y = to<63>(square(op(uy2))) - uy2h;  // u^2 (u^2 - 1)
+    const FxOp<62> A1o = op(to<62>(A1));
+    const Fx<62> ux2h = to<62>(ux2), uy2h = to<62>(uy2);
+    const Fx<62> X = to<62>(square(op(ux2))) - ux2h, Y = to<62>(square(op(uy2))) - uy2h;  // u^2 (u^2 - 1)
     const auto sx = op(c.theta + ux2h), sy = op(c.theta + uy2h);
     const Fx<60> TX = A1o * op(X + c.h), TY = A1o * op(Y + c.h);
-    const Fx<63> px = c.c3 - ux2h, py = uy2h - c.c3;
-    const Fx<60> Ax = A1o * op(px), Ay = A1o * op(py);
+    const Fx<60> Ax = A1o * op(c.c3 - ux2h), Ay = A1o * op(uy2h - c.c3);
     // shear part: omega' N_xy and its products with r_x / theta, r_y / theta
     const Fx<62> nw = op(to<63>(N)) * c.omp;
     const auto nwo = op(nw);
     const Fx<60> vx = c.v0 - op(ux2) * c.inv_theta, vy = c.v0 - op(uy2) * c.inv_theta;
     const auto rx = op(to<62>(ux * op(vx))), ry = op(to<62>(uy * op(vy)));
     const Fx<60> nrx = nwo * rx, nry = nwo * ry;
-    const Fx<60> T20 = rsx + TX, T02 = rsy - TY;
-    M21 = uy * op(T20 + sx * op(to<61>(Ay))) + nrx;
-    M12 = ux * op(T02 + sy * op(to<61>(Ax))) + nry;
-    M22 = op(to<61>(T20)) * sy - op(to<61>(TY)) * sx + op(to<62>(nrx)) * ry;
+    const Fx<60> T20 = rsx + TX, T02 = rsy - TY;  // T20 < 4
+    M21 = uy * op(T20 + sx * op(to<62>(Ay))) + nrx;
+    M12 = ux * op(T02 + sy * op(to<62>(Ax))) + nry;
+    M22 = to<60>(op(to<61>(T20)) * sy - op(to<61>(TY)) * sx) + op(to<62>(nrx)) * ry;
     M11 = jxuy + to<60>(nw);
     if constexpr (MODEL == 1 || MODEL == 2) {
       M20 = T20, M02 = T02;
@@ -344,11 +343,11 @@ OLBM_EMU_HD bool collide(const Moments& m, const Fx<60> (&f)[9], const Coefs& c,
       M22 = M22 - (TX - TY);
     } else {
       const Fx<60> AZ = op(to<64>(TX + TY)) * c.q2;
-      const auto AZo = op(to<61>(AZ));
+      const auto AZo = op(to<62>(AZ));
       const Fx<60> ZX = AZo * op(X + c.t), ZY = AZo * op(Y + c.t);
       M20 = T20 - ZX, M02 = T02 + ZY;
       M22 = M22 - (ZX - ZY);
-      M11 = M11 + op(to<61>(A1 - AZ)) * op(op(ux * uy) * op(uy2h - ux2h));
+      M11 = M11 + op(to<62>(A1 - AZ)) * op(op(ux * uy) * op(uy2h - ux2h));
     }
     if constexpr (MODEL == 1) {  // omega' psi
       M10 = M10 + ux * op(Ax);

@@ -164,9 +164,9 @@ template <typename CT> struct DiagAcc {
     }
   }
 };
-// FP64: nodes of the fixed-point path add into 96-bit integer sums (exact; four
-// 32-bit instructions a sum, where an FP64 addition holds its pipe for 64 cycles),
-// the others into FP64 ones.
+// Forms with FP64 storage: nodes of the fixed-point path add into 96-bit integer sums
+// (exact; four 32-bit instructions a sum, where an FP64 addition holds its pipe for 64
+// cycles), the others into a DiagAcc of the form's arithmetic.
 struct Sum96 {
   unsigned lo = 0, mid = 0;
   int hi = 0;
@@ -181,33 +181,13 @@ struct Sum96 {
     return fma((double)(hi + (int)(mid >> 31)), 16.0, (double)low * 0x1p-60);
   }
 };
-template <> struct DiagAcc<double> {
-  double v[4];
-  int bad;
+struct FixedDiagAcc {
   Sum96 s[4];
-  __device__ DiagAcc() : bad(0) {
-#pragma unroll
-    for (int k = 0; k < 4; ++k) v[k] = 0.0;
-  }
-  __device__ __forceinline__ void add(const NodeMoments<double>& m) {
-    if (finite_lead(m.m0)) {
-      v[0] += m.m0;
-      v[1] += m.jx;
-      v[2] += m.jy;
-      v[3] = fma(m.jx, m.ux, fma(m.jy, m.uy, v[3]));
-    } else {
-      ++bad;
-    }
-  }
   __device__ __forceinline__ void add(const FixedMoments& m) {
     s[0].add(m.rho);
     s[1].add(m.jx);
     s[2].add(m.jy);
     s[3].add(m.ke2);
-  }
-  __device__ __forceinline__ void merge() {
-#pragma unroll
-    for (int k = 0; k < 4; ++k) v[k] += s[k].value();
   }
 };
 // Packed pairs accumulate into four FP32 scalars: both nodes of a pair go into
@@ -239,18 +219,21 @@ template <> struct DiagAcc<f32x2> {
   }
 };
 
-// Reduce a thread's accumulator over the block into out5 (thread 0 writes).
-template <typename CT> __device__ __forceinline__ void block_diag_acc(DiagAcc<CT>& a, double* out5) {
-  if constexpr (std::is_same<CT, double>::value) a.merge();
+// Reduce a thread's accumulators over the block into out5 (thread 0 writes).
+template <typename CT>
+__device__ __forceinline__ void block_diag_acc(DiagAcc<CT>& a, double* out5, const FixedDiagAcc* fixed = nullptr) {
   a.v[3] = scaled(a.v[3], 0.5f);  // kinetic energy
   if constexpr (std::is_same<CT, f32x2>::value) {
     block_diag<float>(a.v, a.bad, out5);
-  } else if constexpr (std::is_same<CT, df64>::value) {
+  } else if constexpr (kHasFixed<CT>) {
     double v[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) v[k] = join_f64(a.v[k]);
+    for (int k = 0; k < 4; ++k) {
+      if constexpr (std::is_same<CT, df64>::value) v[k] = join_f64(a.v[k]);
+      else v[k] = a.v[k];
+      if (fixed != nullptr) v[k] += fixed->s[k].value() * (k == 3 ? 0.5 : 1.0);
+    }
     block_diag<double>(v, a.bad, out5);
-
   } else {
     block_diag<CT>(a.v, a.bad, out5);
   }
@@ -303,37 +286,54 @@ template <int MODEL, int PREC, bool DIAG, bool PAIRS, bool CG = false> struct Co
     }
   }
 
-  // FP64, floating point: the rows r of the column with bit r of `left` set. Out of line:
-  // the rows that the fixed-point collision leaves out are rare, and its registers would
-  // burden the loop that handles the others.
+  // FP64 storage, the form's own arithmetic: the rows r of the column with bit r of
+  // `left` set. Out of line: the rows that the fixed-point collision leaves out are rare,
+  // and its registers would burden the loop that handles the others. The next row's
+  // loads are in flight during the current row's arithmetic (in the double-word form in
+  // the registers of the row just split).
   __device__ static __noinline__ void run_float(const S* __restrict__ src, S* __restrict__ dst, const Geometry& g,
                                                 const Coef<CT>& c, int x, int xm, int xp, int y0, int dy, int rows,
                                                 unsigned long long left, DiagAcc<CT>& acc) {
-    int mode = 0;  // which products this warp's nodes take (see collide)
+    using Raw = Column<MODEL, 0, DIAG, false, CG>;
+    int mode = 0;  // FP64: which products this warp's nodes take (see collide)
+    const unsigned warp = __activemask();
+    double f[9];
+    bool loaded = false;
     for (int r = 0, y = y0; r < rows && y < g.ny; ++r, y += dy) {
       const bool mine = (left >> r) & 1;
-      const unsigned warp = __activemask();
       if (!__any_sync(warp, mine)) continue;
       if (mine) {
-        CT f[9];
-        pull(src, g, x, xm, xp, y, f);
-        collide<MODEL, false, CT>(
-            f, c,
-            [&](const NodeMoments<CT>& m) {
-              if constexpr (DIAG) acc.add(m);
-            },
-            [&](CT (&h)[9]) { pull(src, g, x, xm, xp, y, h); }, &mode);
+        if (!loaded) Raw::pull(src, g, x, xm, xp, y, f);
+        loaded = (r + 1 < rows) && (y + dy < g.ny) && ((left >> (r + 1)) & 1);
         S* q = dst + (long long)y * g.pitch + x;
+        auto sink = [&](const NodeMoments<CT>& m) {
+          if constexpr (DIAG) acc.add(m);
+        };
+        if constexpr (PREC == 3) {
+          df64 d[9];
+          split_node(f, d);
+          if (loaded) Raw::pull(src, g, x, xm, xp, y + dy, f);
+          collide_df<MODEL>(d, c, sink, [&](int i, df64 v) {
+            q[i * g.plane] = kDfJoin == 2 ? join_f64_int(v) : (kDfJoin == 1 ? join_f64_fp64pipe(v) : join_f64(v));
+          });
+        } else if constexpr (PREC == 0) {
+          double fn[9];
+          if (loaded) Raw::pull(src, g, x, xm, xp, y + dy, fn);
+          collide<MODEL, false, double>(
+              f, c, sink, [&](double (&h)[9]) { Raw::pull(src, g, x, xm, xp, y, h); }, &mode);
 #pragma unroll
-        for (int i = 0; i < 9; ++i) st_t(q + i * g.plane, f[i]);
+          for (int i = 0; i < 9; ++i) q[i * g.plane] = f[i], f[i] = fn[i];
+        }
       }
       __syncwarp(warp);
     }
   }
 
+  // FIXED (FP64 storage): the fixed-point collision, which needs c.fixed.on.
+  template <bool FIXED>
   __device__ static __forceinline__ void run(const S* __restrict__ src, S* __restrict__ dst, const Geometry& g,
                                              const Coef<CT>& c, int x, int y0, int dy, int rows,
-                                             DiagAcc<CT>& acc) {
+                                             DiagAcc<CT>& acc, FixedDiagAcc& facc) {
     if (x >= g.nx) return;
     const int xm = (x == 0) ? g.nx - 1 : x - 1;
     int xp;
@@ -342,6 +342,43 @@ template <int MODEL, int PREC, bool DIAG, bool PAIRS, bool CG = false> struct Co
     } else {
       xp = (x == g.nx - 1) ? 0 : x + 1;
     }
+    if constexpr (FIXED) {
+      // The rows in fixed point, the next row's loads going into f once its row is
+      // converted; then the rows it left out (bit r of `left`; rows <= 64) in the form's
+      // own arithmetic.
+      static_assert(PREC == 0 || PREC == 3, "the fixed-point collision is for FP64 storage");
+      using Raw = Column<MODEL, 0, DIAG, false, CG>;
+      unsigned long long left = 0;
+      double f[9];
+      int y = y0;
+      if (y < g.ny) Raw::pull(src, g, x, xm, xp, y, f);
+      for (int r = 0; r < rows && y < g.ny; ++r, y += dy) {
+        double* q = dst + (long long)y * g.pitch + x;
+        const bool done = collide_fixed<MODEL>(
+            f, c.fixed,
+            [&](const FixedMoments& m) {
+              if constexpr (DIAG) facc.add(m);
+            },
+            [&](double (&h)[9]) {
+              if ((r + 1 < rows) && (y + dy < g.ny)) Raw::pull(src, g, x, xm, xp, y + dy, h);
+            },
+            [&](int i, double v) { q[i * g.plane] = v; });
+        left |= done ? 0ull : 1ull << r;
+      }
+      if (__any_sync(__activemask(), left != 0)) {
+        DiagAcc<CT> rest;  // (acc itself stays in registers: its address goes nowhere)
+        run_float(src, dst, g, c, x, xm, xp, y0, dy, rows, left, rest);
+        if constexpr (DIAG) {
+#pragma unroll
+          for (int k = 0; k < 4; ++k) acc.v[k] += rest.v[k];
+          acc.bad += rest.bad;
+        }
+      }
+      return;
+    }
+    auto sink = [&](const NodeMoments<CT>& m) {
+      if constexpr (DIAG) acc.add(m);
+    };
     if constexpr (PREC == 3) {
       // Double-word form: the loads stay raw FP64 until their row is computed,
       // so the next row's loads are in flight during the current row's arithmetic
@@ -357,58 +394,21 @@ template <int MODEL, int PREC, bool DIAG, bool PAIRS, bool CG = false> struct Co
         // flight during this row's collision (no second set of registers).
         if ((k + 1 < rows) && (y + dy < g.ny)) Raw::pull(src, g, x, xm, xp, y + dy, r);
         S* q = dst + (long long)y * g.pitch + x;
-        collide_df<MODEL>(
-            f, c,
-            [&](const NodeMoments<df64>& m) {
-              if constexpr (DIAG) acc.add(m);
-            },
-            [&](int i, df64 v) {
-              q[i * g.plane] = kDfJoin == 2 ? join_f64_int(v) : (kDfJoin == 1 ? join_f64_fp64pipe(v) : join_f64(v));
-            });
-      }
-      return;
-    }
-    auto sink = [&](const auto& m) {
-      if constexpr (DIAG) acc.add(m);
-    };
-    if constexpr (PREC == 0) {
-      // FP64: the rows in fixed point, the next row's loads going into f once its row is
-      // converted; then the rows it left out (bit r of `left`; rows <= 64) in floating point.
-      unsigned long long left = ~0ull;
-      if (c.fixed.on) {
-        left = 0;
-        double f[9];
-        int y = y0;
-        if (y < g.ny) pull(src, g, x, xm, xp, y, f);
-        for (int r = 0; r < rows && y < g.ny; ++r, y += dy) {
-          double* q = dst + (long long)y * g.pitch + x;
-          const bool done = collide_fixed<MODEL>(
-              f, c, sink,
-              [&](double (&h)[9]) {
-                if ((r + 1 < rows) && (y + dy < g.ny)) pull(src, g, x, xm, xp, y + dy, h);
-              },
-              [&](int i, double v) { q[i * g.plane] = v; });
-          left |= done ? 0ull : 1ull << r;
-        }
-      }
-      if (__any_sync(__activemask(), left != 0)) {
-        DiagAcc<CT> rest;  // (acc itself stays in registers: its address goes nowhere)
-        run_float(src, dst, g, c, x, xm, xp, y0, dy, rows, left, rest);
-        if constexpr (DIAG) {
-#pragma unroll
-          for (int k = 0; k < 4; ++k) acc.v[k] += rest.v[k];
-          acc.bad += rest.bad;
-        }
+        collide_df<MODEL>(f, c, sink, [&](int i, df64 v) {
+          q[i * g.plane] = kDfJoin == 2 ? join_f64_int(v) : (kDfJoin == 1 ? join_f64_fp64pipe(v) : join_f64(v));
+        });
       }
       return;
     }
     CT f[9], fn[9];
     int y = y0;
+    int mode = 0;  // FP64: which products this warp's nodes take (see collide)
     if (y < g.ny) pull(src, g, x, xm, xp, y, f);
     for (int r = 0; r < rows && y < g.ny; ++r, y += dy) {
       const bool more = (r + 1 < rows) && (y + dy < g.ny);
       if (more) pull(src, g, x, xm, xp, y + dy, fn);
-      collide<MODEL, Form<PREC>::kShift, CT>(f, c, sink);
+      collide<MODEL, Form<PREC>::kShift, CT>(
+          f, c, sink, [&](CT (&h)[9]) { pull(src, g, x, xm, xp, y, h); }, &mode);
       S* q = dst + (long long)y * g.pitch + x;
       if constexpr (PAIRS) {
 #pragma unroll
@@ -430,7 +430,7 @@ template <int MODEL, int PREC, bool DIAG, bool PAIRS, bool CG = false> struct Co
 // With DIAG, per-block sums of mass (as the stored deviation m0), momentum,
 // kinetic energy and the number of nodes whose pulled populations do not sum to
 // a finite value go to partials[block * 5 + k].
-template <int MODEL, int PREC, bool DIAG, bool PAIRS>
+template <int MODEL, int PREC, bool DIAG, bool PAIRS, bool FIXED = false>
 __device__ __forceinline__ void step_body(const typename Form<PREC>::S* __restrict__ src,
                                           typename Form<PREC>::S* __restrict__ dst, const Geometry& g,
                                           const Coef<typename Column<MODEL, PREC, DIAG, PAIRS>::CT>& c,
@@ -440,31 +440,34 @@ __device__ __forceinline__ void step_body(const typename Form<PREC>::S* __restri
   const int x = PAIRS ? 2 * t : t;
   const int y0 = blockIdx.y * blockDim.y * rows + threadIdx.y;
   DiagAcc<typename Col::CT> acc;
-  Col::run(src, dst, g, c, x, y0, (int)blockDim.y, rows, acc);
-  if constexpr (DIAG) block_diag_acc(acc, partials + (long long)(blockIdx.y * gridDim.x + blockIdx.x) * 5);
+  FixedDiagAcc facc;
+  Col::template run<FIXED>(src, dst, g, c, x, y0, (int)blockDim.y, rows, acc, facc);
+  if constexpr (DIAG)
+    block_diag_acc(acc, partials + (long long)(blockIdx.y * gridDim.x + blockIdx.x) * 5, &facc);
 }
 
-template <int MODEL, int PREC, bool DIAG, bool PAIRS>
+template <int MODEL, int PREC, bool DIAG, bool PAIRS, bool FIXED = false>
 __global__ void __launch_bounds__(512) step_kernel(const typename Form<PREC>::S* __restrict__ src,
                                                    typename Form<PREC>::S* __restrict__ dst, Geometry g,
                                                    Coef<typename Column<MODEL, PREC, DIAG, PAIRS>::CT> c,
                                                    double* __restrict__ partials, int rows) {
-  step_body<MODEL, PREC, DIAG, PAIRS>(src, dst, g, c, partials, rows);
+  step_body<MODEL, PREC, DIAG, PAIRS, FIXED>(src, dst, g, c, partials, rows);
 }
 
-// Double-word form (3): launched with at most 256 threads a block and capped
-// at 96 registers a thread, five blocks of 128 threads per SM. The complete
-// model with fused diagnostics at 4096^2 (integer join): 80, 88 and 96
-// registers give 24.7, 25.0 and 25.2 GLUPS (80 spills 48 bytes); uncapped it
-// takes more than 100 registers and four blocks per SM.
+// Double-word form (3): the fixed-point collision (FIXED) in the same loop as the FP64
+// form's, double-word arithmetic for the nodes outside its range and for temperatures it
+// does not take. Launched with at most 256 threads a block and capped at 96 registers a
+// thread, five blocks of 128 threads per SM. The complete model with fused diagnostics at
+// 4096^2: 30.8 GLUPS (25.2 with every node in double-word arithmetic; that with 80 and 88
+// registers 24.7 and 25.0).
 #ifndef OLBM_DF_MAXNREG
 #define OLBM_DF_MAXNREG 96
 #endif
-template <int MODEL, bool DIAG, bool PAIRS>
+template <int MODEL, bool DIAG, bool FIXED>
 __global__ void __maxnreg__(OLBM_DF_MAXNREG) step_kernel_df(const double* __restrict__ src, double* __restrict__ dst,
-                                                      Geometry g, Coef<typename Column<MODEL, 3, DIAG, PAIRS>::CT> c,
+                                                      Geometry g, Coef<df64> c,
                                                       double* __restrict__ partials, int rows) {
-  step_body<MODEL, 3, DIAG, PAIRS>(src, dst, g, c, partials, rows);
+  step_body<MODEL, 3, DIAG, false, FIXED>(src, dst, g, c, partials, rows);
 }
 
 // The FP64 form collides in 64-bit fixed point on the integer pipes (lbm_fixed.cuh),
@@ -480,6 +483,16 @@ __global__ void __maxnreg__(OLBM_DF_MAXNREG) step_kernel_df(const double* __rest
 template <int MODEL, bool DIAG>
 __global__ void __maxnreg__(OLBM_F64_MAXNREG) step_kernel_f64(const double* __restrict__ src, double* __restrict__ dst, Geometry g,
                                                 Coef<double> c, double* __restrict__ partials, int rows) {
+  step_body<MODEL, 0, DIAG, false, true>(src, dst, g, c, partials, rows);
+}
+
+// The FP64 form for temperatures and relaxation times that the fixed-point formats do not
+// take: bound by the FP64 pipe, its products on the integer pipes. Capped at 128 registers
+// (four blocks of 128 threads an SM, a few bytes spilled): 6.33 GLUPS at 4096^2.
+template <int MODEL, bool DIAG>
+__global__ void __maxnreg__(128) step_kernel_f64_float(const double* __restrict__ src, double* __restrict__ dst,
+                                                       Geometry g, Coef<double> c, double* __restrict__ partials,
+                                                       int rows) {
   step_body<MODEL, 0, DIAG, false>(src, dst, g, c, partials, rows);
 }
 
@@ -709,19 +722,13 @@ template <int PREC> struct Launch {
     const dim3 grid = step_grid(a.g, a.cfg, PREC);
     if constexpr (PREC == 3) {
       if (block.x * block.y > 256) return cudaErrorInvalidConfiguration;
-      if (a.diag)
-        step_kernel_df<MODEL, true, PAIRS><<<grid, block, 0, st>>>((const S*)a.src, (S*)a.dst, a.g, c, a.partials,
-                                                                    a.cfg.rows);
-      else
-        step_kernel_df<MODEL, false, PAIRS><<<grid, block, 0, st>>>((const S*)a.src, (S*)a.dst, a.g, c, a.partials,
-                                                                     a.cfg.rows);
+      auto kernel = c.fixed.on ? (a.diag ? step_kernel_df<MODEL, true, true> : step_kernel_df<MODEL, false, true>)
+                               : (a.diag ? step_kernel_df<MODEL, true, false> : step_kernel_df<MODEL, false, false>);
+      kernel<<<grid, block, 0, st>>>((const S*)a.src, (S*)a.dst, a.g, c, a.partials, a.cfg.rows);
     } else if constexpr (PREC == 0) {
-      if (a.diag)
-        step_kernel_f64<MODEL, true><<<grid, block, 0, st>>>((const S*)a.src, (S*)a.dst, a.g, c, a.partials,
-                                                              a.cfg.rows);
-      else
-        step_kernel_f64<MODEL, false><<<grid, block, 0, st>>>((const S*)a.src, (S*)a.dst, a.g, c, a.partials,
-                                                               a.cfg.rows);
+      auto kernel = c.fixed.on ? (a.diag ? step_kernel_f64<MODEL, true> : step_kernel_f64<MODEL, false>)
+                               : (a.diag ? step_kernel_f64_float<MODEL, true> : step_kernel_f64_float<MODEL, false>);
+      kernel<<<grid, block, 0, st>>>((const S*)a.src, (S*)a.dst, a.g, c, a.partials, a.cfg.rows);
     } else {
       if (a.diag)
         step_kernel<MODEL, PREC, true, PAIRS><<<grid, block, 0, st>>>((const S*)a.src, (S*)a.dst, a.g, c, a.partials,

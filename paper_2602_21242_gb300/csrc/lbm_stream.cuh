@@ -340,7 +340,7 @@ template <int PREC, int NC, int STAGES> struct Pipeline {
   template <int MODEL, bool DIAG>
   __device__ __forceinline__ bool consume_f64(double* __restrict__ dst, const Geometry& g, const Coef<double>& c,
                                               int x0, int y0, int rows, int t, int lane, DiagAcc<double>& acc,
-                                              int* err) {
+                                              FixedDiagAcc& facc, int* err) {
     static_assert(PREC == 0, "one node a consumer thread is the FP64 layout");
     const TilePlan<CH> p(g, x0, W, SEG);
     const int j = t / p.w;
@@ -371,16 +371,23 @@ template <int PREC, int NC, int STAGES> struct Pipeline {
       if (lane == 0) mbar_arrive(&empty[s]);
       if (active) {
         double* q = dst + (long long)(y0 + r0 + j) * g.pitch + x0 + xl;
-        auto sink = [&](const auto& m) {
-          if constexpr (DIAG) acc.add(m);
-        };
         auto store = [&](int i, double v) { q[i * g.plane] = v; };
         double h[9];
 #pragma unroll
         for (int i = 0; i < 9; ++i) h[i] = f[i];
-        const bool left = !c.fixed.on || !collide_fixed<MODEL>(h, c, sink, [](double (&)[9]) {}, store);
+        const bool left = !c.fixed.on || !collide_fixed<MODEL>(
+                                               h, c.fixed,
+                                               [&](const FixedMoments& m) {
+                                                 if constexpr (DIAG) facc.add(m);
+                                               },
+                                               [](double (&)[9]) {}, store);
         if (__any_sync(__activemask(), left) && left) {
-          collide<MODEL, false, double>(f, c, sink, KeepInputs(), &mode);
+          collide<MODEL, false, double>(
+              f, c,
+              [&](const NodeMoments<double>& m) {
+                if constexpr (DIAG) acc.add(m);
+              },
+              KeepInputs(), &mode);
 #pragma unroll
           for (int i = 0; i < 9; ++i) store(i, f[i]);
         }
@@ -507,14 +514,16 @@ __global__ void __launch_bounds__(NC + 32, 4) step_stream_f64_kernel(const doubl
   const int rows = min(H, g.ny - y0);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   DiagAcc<double> acc;
+  FixedDiagAcc facc;
   if (warp == P::kConsumerWarps) {
     pdl_wait();
     pipe.produce(src, g, x0, y0, rows, lane, err);
     pipe.drain(err);
   } else if (threadIdx.x < NC) {
-    pipe.template consume_f64<MODEL, DIAG>(dst, g, c, x0, y0, rows, threadIdx.x, lane, acc, err);
+    pipe.template consume_f64<MODEL, DIAG>(dst, g, c, x0, y0, rows, threadIdx.x, lane, acc, facc, err);
   }
-  if constexpr (DIAG) block_diag_acc(acc, partials + (long long)(blockIdx.y * gridDim.x + blockIdx.x) * 5);
+  if constexpr (DIAG)
+    block_diag_acc(acc, partials + (long long)(blockIdx.y * gridDim.x + blockIdx.x) * 5, &facc);
 }
 
 }  // namespace olbm

@@ -35,7 +35,7 @@ def _rows(checker, n, theta, tau):
     return [[float(v) for v in line.split()] for line in out.stdout.splitlines()]
 
 
-@pytest.mark.parametrize("theta,tau", [(0.21, 0.501), (0.25, 3.0), (1 / 3, 0.515), (0.4, 0.55), (0.5, 1.0), (0.57, 50.0)])
+@pytest.mark.parametrize("theta,tau", [(0.21, 0.501), (0.25, 3.0), (1 / 3, 0.515), (0.4, 0.55), (0.5, 1.0), (0.57, 50.0), (0.65, 0.6)])
 def test_error_against_extended_precision(checker, theta, tau):
     rows = _rows(checker, 20_000, theta, tau)
     assert len(rows) == 24
@@ -45,6 +45,6 @@ def test_error_against_extended_precision(checker, theta, tau):
         assert rms <= max(rms64, 1.01 * rounding), (model, family, rms, rms64, rounding)
 
 
-@pytest.mark.parametrize("theta,tau", [(0.2, 0.8), (0.6, 0.8), (1 / 3, 1e12)])
+@pytest.mark.parametrize("theta,tau", [(0.2, 0.8), (0.66, 0.8), (1 / 3, 1e12)])
 def test_coefficients_outside_the_range_are_left_out(checker, theta, tau):
     assert all(row[3] == 0 for row in _rows(checker, 100, theta, tau))

@@ -32,7 +32,7 @@ def _state(oracle, nx, ny, theta, seed):
     return np.ascontiguousarray(f)
 
 
-@pytest.mark.parametrize("theta", [0.15, 0.21, 1 / 3, 0.57, 0.65])
+@pytest.mark.parametrize("theta", [0.15, 0.21, 1 / 3, 0.65, 0.7])
 @pytest.mark.parametrize("model", [0, 1, 2, 3, 4, 5])
 def test_both_paths_of_one_step(oracle, model, theta):
     nx, ny, tau = 150, 37, 0.77
