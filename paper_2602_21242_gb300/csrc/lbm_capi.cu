@@ -15,6 +15,7 @@
 #include "lbm.h"
 #include "lbm_ctx.h"
 #include "lbm_launch.h"
+#include "lbm_tile.h"
 #include "lbm_halo.h"
 #include "lbm_walls.h"
 
@@ -54,13 +55,14 @@ bool layout_of(int nx, int ny, int prec, long long* pitch, long long* plane, lon
 
 long long nodes_of(const lbm_ctx* c) { return (long long)c->nx * c->ny; }
 
-// Default launch of the step kernel per storage form, chosen by timing on GB300
-// at the 4096^2 benchmark size: FP64 the column kernel with 64 x 2 threads and
-// 32 rows per thread; the shifted forms the bulk-copy pipeline with one CTA per
-// tile of 32 rows (refined per form below), except on lattices narrower than 32
-// columns, where the column kernel with 128 x 4 threads and 16 rows wastes fewer
-// threads. On smaller lattices the rows are halved until the grid has at least
-// 4 CTAs per SM.
+// Default launch of the step kernel per storage form, chosen by timing on GB300:
+// FP64 storage the column kernel with 64 x 2 threads and up to 32 rows per thread, fewer
+// on smaller lattices so that the grid has at least 20 CTAs per SM (four waves of the five
+// resident: 2048^2 6 to 10 rows 125-126 us a step, 32 rows 136; 1531 x 1277 2 to 6 rows
+// 61.6, 16 rows 69.6; diagnosed steps take more rows, see diag_rows); the shifted forms the bulk-copy pipeline with one CTA per tile of 32
+// rows (refined per form below), except on lattices narrower than 32 columns, where the
+// column kernel with 128 x 4 threads and 16 rows wastes fewer threads. On smaller lattices
+// their rows are halved until the grid has at least 4 CTAs per SM.
 // lbm_set_launch[_ex] (and the autotuner built on it) overrides the choice.
 olbm::LaunchCfg default_cfg(int prec, const olbm::Geometry& g, int sms) {
   olbm::LaunchCfg k;
@@ -85,7 +87,11 @@ olbm::LaunchCfg default_cfg(int prec, const olbm::Geometry& g, int sms) {
       if (waste < best_waste - 0.02) best_waste = waste, k.rows = rows;
     }
   }
-  while (k.rows > 1 && olbm::step_blocks(g, k, prec) < 4LL * sms) k.rows /= 2;
+  if (prec == LBM_F64 || prec == LBM_F64_DF) {
+    while (k.rows > 1 && olbm::step_blocks(g, k, prec) < 20LL * sms) --k.rows;
+  } else {
+    while (k.rows > 1 && olbm::step_blocks(g, k, prec) < 4LL * sms) k.rows /= 2;
+  }
   // FP32: two steps a launch (kind 2) on 24-row tiles, 48 from 8192^2 (diagnostics
   // every step: 143.6 GLUPS at 4096^2 against 92.6 for single steps, heights 16 to
   // 58 within 3 %; 161.6 at 8192^2 against 96.7); where it does not apply, the persistent pipeline over all
@@ -96,12 +102,26 @@ olbm::LaunchCfg default_cfg(int prec, const olbm::Geometry& g, int sms) {
     olbm::LaunchCfg k2 = k;
     k2.kind = 2, k2.bx = 0, k2.rows = g.nx >= 8192 && g.ny >= 8192 ? 48 : 24;
     if (olbm::uses_step2(prec, g, k2)) {
-      while (k2.rows > 1 && olbm::step2_blocks(g, k2, prec) < 4LL * sms) k2.rows /= 2;
+      // Smaller lattices (four CTAs an SM resident): the rows that make one wave while those
+      // are few, else those that make at least two (us a step: 512^2 3 rows 5.1, 1 row 7.4;
+      // 768^2 6 rows 7.8, 3 rows 8.6; 1536^2 8 rows 21.7, 16 rows 23.5; 2048^2 12 to 16 rows
+      // 33.2 to 33.6, 24 rows 37.6).
+      const long long wave = 4LL * sms, strips = (g.nx + olbm::step2_tile_width(prec) - 1) / olbm::step2_tile_width(prec);
+      const long long one = (strips * g.ny + wave - 1) / wave, two = strips * g.ny / (2 * wave);
+      k2.rows = (int)std::max<long long>(1, std::min<long long>(k2.rows, one <= 9 ? one : two));
       return k2;
     }
     k.bx = 64, k.rows = k.rows < 4 ? k.rows : 4;
   }
   return k;
+}
+
+// Rows per thread of a diagnosed FP64 step under the default launch: at least 6 CTAs per SM
+// where the plain step has 20, because one block sums the CTAs' partials beside the next
+// step (512^2, diagnostics every step: 37.0 us a step with 1 row and 4096 partials).
+int diag_rows(const olbm::Geometry& g, olbm::LaunchCfg k, int prec, int sms) {
+  for (k.rows = 32; k.rows > 1 && olbm::step_blocks(g, k, prec) < 6LL * sms;) --k.rows;
+  return k.rows;
 }
 
 cudaError_t launch_step(const olbm::StepArgs& a, int prec, cudaStream_t st) {
@@ -118,6 +138,15 @@ cudaError_t launch_step2(const olbm::StepArgs& a, int prec, cudaStream_t st) {
     case LBM_F32_SHIFT: return olbm::launch_step2_f32(a, st);
     case LBM_F16_SHIFT: return olbm::launch_step2_f16(a, st);
     default: return cudaErrorInvalidValue;
+  }
+}
+
+cudaError_t launch_tile(const olbm::StepArgs& a, const olbm::TilesPlan& p, int steps, int prec, cudaStream_t st) {
+  switch (prec) {
+    case LBM_F64: return olbm::launch_tile_f64(a, p, steps, st);
+    case LBM_F32_SHIFT: return olbm::launch_tile_f32(a, p, steps, st);
+    case LBM_F64_DF: return olbm::launch_tile_f64df(a, p, steps, st);
+    default: return olbm::launch_tile_f16(a, p, steps, st);
   }
 }
 
@@ -161,6 +190,7 @@ void free_ctx(lbm_ctx* c) {
   cudaFree(c->d_stage);
   cudaFree(c->d_vjp);
   cudaFree(c->d_walls);
+  cudaFree(c->d_wall_mask);
   delete c;
 }
 
@@ -217,7 +247,14 @@ int lbm_create_ex(int nx, int ny, double theta, double tau, int model, int prec,
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess || sms < 1) sms = 1;
   c->cfg = default_cfg(prec, c->g, sms);
   c->nparts = olbm::step_blocks(c->g, c->cfg, prec);
-  c->parts_cap = std::max(c->nparts, olbm::node_blocks(c->g));
+  if (prec == LBM_F64 || prec == LBM_F64_DF) c->diag_rows = diag_rows(c->g, c->cfg, prec, sms);
+  // FP32 / FP16 lattices with an odd width below 32 columns update single nodes (kind 0),
+  // whose last bits differ from the node pairs of the tiles: they keep single steps.
+  if (c->cfg.kind != 0 || prec == LBM_F64 || prec == LBM_F64_DF || nx % 2 == 0)
+    for (int w = 0; w < 2; ++w) c->tile[w] = olbm::tile_plan(c->g, prec, theta, tau, sms, w != 0);
+  // (a cut into tiles has at most two an SM)
+  // (diagnosed steps take at least as many rows, so no more partials, unless one row is all there is)
+  c->parts_cap = std::max({c->nparts, olbm::node_blocks(c->g), 2LL * sms});
 
   if (d_pop_buffers) {
     c->own_buffers = false;
@@ -345,17 +382,25 @@ int lbm_set_walls(lbm_ctx* ctx, const unsigned char* h_mask, long long* h_count)
     return cuda_fail(ctx, e, "lbm_set_walls sync");
   }
   cudaFree(ctx->d_walls);
+  cudaFree(ctx->d_wall_mask);
   ctx->d_walls = nullptr;
+  ctx->d_wall_mask = nullptr;
   ctx->n_walls = 0;
   if (n > 0) {
     e = cudaMalloc(&ctx->d_walls, sizeof(int2) * (size_t)n);
     if (e == cudaSuccess)
       e = cudaMemcpy(ctx->d_walls, list, sizeof(int2) * (size_t)n, cudaMemcpyHostToDevice);
     delete[] list;
+    if (e == cudaSuccess && ctx->tile[1].on()) {
+      e = cudaMalloc(&ctx->d_wall_mask, (size_t)nodes);
+      if (e == cudaSuccess) e = cudaMemcpy(ctx->d_wall_mask, h_mask, (size_t)nodes, cudaMemcpyHostToDevice);
+    }
     if (e != cudaSuccess) {
       cudaGetLastError();
       cudaFree(ctx->d_walls);
+      cudaFree(ctx->d_wall_mask);
       ctx->d_walls = nullptr;
+      ctx->d_wall_mask = nullptr;
       return fail(ctx, e == cudaErrorMemoryAllocation ? LBM_ENOMEM : LBM_ECUDA, "lbm_set_walls: %s",
                   cudaGetErrorString(e));
     }
@@ -463,23 +508,36 @@ int lbm_step(lbm_ctx* ctx, int n) {
     return cudaSuccess;
   };
   auto due = [&](long long t) { return ctx->diag_every > 0 && (t % ctx->diag_every) == 0; };
+  a.wall_mask = ctx->d_wall_mask;
   for (int k = 0; k < n;) {
+    // Small lattices: several steps in one launch, as many as remain before the next diagnosed
+    // step (only the first step of a launch is diagnosed).
+    int many = 1;
+    const olbm::TilesPlan& tile = ctx->tile[ctx->n_walls > 0 ? 1 : 0];
+    if (tile.on()) {
+      const long long next = ctx->diag_every > 0 ? ctx->diag_every - ctx->t % ctx->diag_every : n;
+      many = (int)std::min<long long>({tile.steps, n - k, next});
+    }
     // launch kind 2: two steps in one launch where two remain (no walls: they act after every step)
-    const bool two = k + 1 < n && ctx->n_walls == 0 && olbm::uses_step2(ctx->prec, ctx->g, ctx->cfg);
+    const bool two = many < 2 && k + 1 < n && ctx->n_walls == 0 && olbm::uses_step2(ctx->prec, ctx->g, ctx->cfg);
     a.diag = due(ctx->t);
     a.diag2 = two && due(ctx->t + 1);
     a.src = ctx->buf[ctx->cur];
     a.dst = ctx->buf[ctx->cur ^ 1];
     used = ctx->nparts;
+    a.cfg.rows = a.diag && ctx->diag_rows > 0 ? ctx->diag_rows : ctx->cfg.rows;
+    if (a.cfg.rows != ctx->cfg.rows) used = olbm::step_blocks(ctx->g, a.cfg, ctx->prec);
     int b1 = -1, b2 = -1;
     cudaError_t e = take(a.diag, b1);
     if (e == cudaSuccess) e = take(a.diag2, b2);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "lbm_step event wait");
     a.partials = ctx->d_parts[b1 < 0 ? 0 : b1];
     a.partials2 = ctx->d_parts[b2 < 0 ? 0 : b2];
-    e = two ? launch_step2(a, ctx->prec, ctx->stream) : launch_step(a, ctx->prec, ctx->stream);
+    e = many > 1 ? launch_tile(a, tile, many, ctx->prec, ctx->stream)
+        : two    ? launch_step2(a, ctx->prec, ctx->stream)
+                 : launch_step(a, ctx->prec, ctx->stream);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "lbm_step launch");
-    if (ctx->n_walls > 0) {
+    if (ctx->n_walls > 0 && many < 2) {
       e = olbm::launch_walls((int)elem_size(ctx->prec), a.src, a.dst, ctx->g, ctx->d_walls, ctx->n_walls,
                              ctx->stream);
       if (e != cudaSuccess) return cuda_fail(ctx, e, "lbm_step walls launch");
@@ -488,7 +546,7 @@ int lbm_step(lbm_ctx* ctx, int n) {
     if (b2 >= 0 && (e = finish(b2, ctx->t + 1)) != cudaSuccess)
       return cuda_fail(ctx, e, "lbm_step diagnostics launch");
     ctx->cur ^= 1;
-    const int done = two ? 2 : 1;
+    const int done = many > 1 ? many : (two ? 2 : 1);
     ctx->t += done;
     k += done;
   }
@@ -684,6 +742,8 @@ int lbm_set_launch_ex(lbm_ctx* ctx, int kind, int bx, int by, int rows) {
     ctx->parts_cap = need;
   }
   ctx->cfg = k;
+  ctx->diag_rows = 0;
+  ctx->tile[0] = ctx->tile[1] = olbm::TilesPlan{};  // the chosen shape, nothing else
   ctx->nparts = need;
   return LBM_OK;
 }

@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 
 #include "lbm_launch.h"
+#include "lbm_tile.h"
 
 struct lbm_ctx {
   int device = 0;
@@ -18,6 +19,9 @@ struct lbm_ctx {
   bool initialised = false;
   cudaStream_t stream = nullptr;
   olbm::LaunchCfg cfg{};
+  int diag_rows = 0;  // rows of a diagnosed step under the default FP64 launch (0: as cfg)
+  // several steps a launch on small lattices, without and with walls; off once lbm_set_launch chose a shape
+  olbm::TilesPlan tile[2]{};
   // Per-block diagnostics partials, kParts buffers of parts_cap blocks each (d_parts[0]
   // also serves lbm_diagnostics). Consecutive diagnosed steps take the buffers in turn,
   // and the final sum of step t runs on a second stream while later steps run; lbm_step
@@ -55,6 +59,7 @@ struct lbm_ctx {
   // fullway bounce-back wall nodes (x, y), applied after every step (lbm_set_walls)
   int2* d_walls = nullptr;
   long long n_walls = 0;
+  unsigned char* d_wall_mask = nullptr;  // nx * ny bytes, where tile[1] is used and walls are set
   // Slab halo trade (lbm_halo_pack / lbm_halo_unpack): the time of the last
   // unpack, or of lbm_init / lbm_set_state (a pack needs exactly one step
   // since), and the time of the last pack (an unpack needs one at this time).

@@ -41,6 +41,26 @@ constexpr int kDiagRows = 8;  // rows per thread of the diagnostics kernel (one 
 // 25.2 with 2.
 constexpr int kDfJoin = OLBM_DF_JOIN;
 
+// Programmatic dependent launch (sm_90 and later). A step kernel launched with
+// the programmatic-serialization attribute may be scheduled while the previous
+// kernel of its stream is finishing; every CTA of a step kernel signals that the
+// next grid may launch (launch_dependents), and the next grid waits for the
+// previous grid to complete, its writes visible, before it touches anything that
+// grid read or wrote (griddepcontrol.wait, a no-op for a kernel launched without
+// the attribute). What overlaps is the next grid's launch and set-up with the
+// previous grid's last CTAs. The bulk-copy kernels signal at their start (their
+// producer waits, their consumers touch global memory only after its copies); the
+// kernels that load through L1 signal after their own wait, so that no grid
+// before the previous one is still reading when the next one starts, and use plain
+// loads (the read-only path is not for data written while a grid is resident).
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ double ld_plain(const double* p) {
+  double v;
+  asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
+  return v;
+}
+
 // Source offsets of the pull f_i(x) = B_i(x - c_i) inside one plane.
 __device__ __forceinline__ void pull_offsets(int x, int y, const Geometry& g, long long (&o)[9]) {
   const int xm = (x == 0) ? g.nx - 1 : x - 1;
@@ -273,7 +293,11 @@ template <int MODEL, int PREC, bool DIAG, bool PAIRS, bool CG = false> struct Co
       f[8] = T2(pp + 8 * g.plane + xm, pp + 8 * g.plane + x);
     } else {
       // xm = x - 1, xp = x + 1 (periodic)
-      auto L = [](const S* q) { return CG ? ld_cg(q, CT()) : ld_t(q, CT()); };
+      auto L = [](const S* q) {
+        if constexpr (CG) return ld_cg(q, CT());
+        else if constexpr (PREC == 0) return ld_plain(q);
+        else return ld_t(q, CT());
+      };
       f[0] = L(p0 + x);
       f[1] = L(p0 + 1 * g.plane + xm);
       f[2] = L(pm + 2 * g.plane + x);
@@ -441,6 +465,10 @@ __device__ __forceinline__ void step_body(const typename Form<PREC>::S* __restri
   const int y0 = blockIdx.y * blockDim.y * rows + threadIdx.y;
   DiagAcc<typename Col::CT> acc;
   FixedDiagAcc facc;
+  if constexpr (PREC == 0 || PREC == 3) {  // launched with programmatic serialization
+    pdl_wait();
+    pdl_launch_dependents();
+  }
   Col::template run<FIXED>(src, dst, g, c, x, y0, (int)blockDim.y, rows, acc, facc);
   if constexpr (DIAG)
     block_diag_acc(acc, partials + (long long)(blockIdx.y * gridDim.x + blockIdx.x) * 5, &facc);
@@ -724,11 +752,11 @@ template <int PREC> struct Launch {
       if (block.x * block.y > 256) return cudaErrorInvalidConfiguration;
       auto kernel = c.fixed.on ? (a.diag ? step_kernel_df<MODEL, true, true> : step_kernel_df<MODEL, false, true>)
                                : (a.diag ? step_kernel_df<MODEL, true, false> : step_kernel_df<MODEL, false, false>);
-      kernel<<<grid, block, 0, st>>>((const S*)a.src, (S*)a.dst, a.g, c, a.partials, a.cfg.rows);
+      return launch_step_kernel(kernel, grid, block, 0, st, (const S*)a.src, (S*)a.dst, a.g, c, a.partials, a.cfg.rows);
     } else if constexpr (PREC == 0) {
       auto kernel = c.fixed.on ? (a.diag ? step_kernel_f64<MODEL, true> : step_kernel_f64<MODEL, false>)
                                : (a.diag ? step_kernel_f64_float<MODEL, true> : step_kernel_f64_float<MODEL, false>);
-      kernel<<<grid, block, 0, st>>>((const S*)a.src, (S*)a.dst, a.g, c, a.partials, a.cfg.rows);
+      return launch_step_kernel(kernel, grid, block, 0, st, (const S*)a.src, (S*)a.dst, a.g, c, a.partials, a.cfg.rows);
     } else {
       if (a.diag)
         step_kernel<MODEL, PREC, true, PAIRS><<<grid, block, 0, st>>>((const S*)a.src, (S*)a.dst, a.g, c, a.partials,

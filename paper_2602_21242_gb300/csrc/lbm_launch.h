@@ -46,6 +46,7 @@ struct StepArgs {
   // two-step launches (kind 2): diagnostics of the second step into partials2
   bool diag2 = false;
   double* partials2 = nullptr;
+  const unsigned char* wall_mask = nullptr;  // several-steps-a-launch tiles: nonzero = wall node, or NULL
 };
 
 // Number of thread blocks of the auxiliary node-parallel kernels and of the
@@ -58,6 +59,8 @@ long long step_blocks(const Geometry& g, const LaunchCfg& k, int prec);
 // on one SM (launch kind 1) for a shifted storage form.
 int stream_tile_width(int prec);
 int stream_ctas_per_sm(int prec);
+// Output columns of a two-step tile (launch kind 2).
+int step2_tile_width(int prec);
 // Whether a launch of kind 2 runs two steps (the shifted forms), and
 // the blocks (= diagnostics partials) of that two-step launch.
 bool uses_step2(int prec, const Geometry& g, const LaunchCfg& k);

@@ -25,6 +25,8 @@ long long step_blocks(const Geometry& g, const LaunchCfg& k, int prec) {
 
 int stream_tile_width(int prec) { return stream_width(prec); }
 
+int step2_tile_width(int prec) { return stream2_width(prec); }
+
 bool uses_step2(int prec, const Geometry& g, const LaunchCfg& k) { return step2_applies(prec, g, k); }
 
 long long step2_blocks(const Geometry& g, const LaunchCfg& k, int prec) {
@@ -42,7 +44,7 @@ int stream_ctas_per_sm(int) { return OLBM_STREAM_CTAS; }
 // Fixed-order final sum of the block partials: out[0..4] as in lbm_diagnostics
 // (mass gets rho_ref for every finite node), out[5] = t; non-finite nodes are
 // added to *sticky.
-constexpr int kFinalThreads = 256;
+constexpr int kFinalThreads = 512;
 __global__ void __launch_bounds__(kFinalThreads) finalize_kernel(const double* __restrict__ partials, int nparts,
                                                                  double rho_ref, long long nodes, long long t,
                                                                  double* __restrict__ out,

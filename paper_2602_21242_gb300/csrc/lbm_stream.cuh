@@ -69,19 +69,6 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, unsigned by
       : "memory");
 }
 
-// Programmatic dependent launch (sm_90 and later). A step kernel launched with
-// the programmatic-serialization attribute may be scheduled while the previous
-// kernel of its stream is finishing; every CTA of a step kernel signals at its
-// start that the next grid may launch (launch_dependents), and the next grid's
-// producer waits for the previous grid to complete, its writes visible, before
-// it reads anything that grid wrote (griddepcontrol.wait, a no-op for a kernel
-// launched without the attribute). The consumers touch global memory only
-// after the producer's copies, so they follow the wait. What overlaps is the
-// next grid's launch and set-up (CTA placement, mbarrier initialisation) with
-// the previous grid's last CTAs.
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
 // Grid barrier with bounded waits. count/gen/err live in device memory zeroed
 // before the launch. Returns false (in every thread of the block) once any
 // block has given up.
