@@ -97,6 +97,8 @@ struct lbm_batch {
   int4* d_tiles = nullptr;
   int2* d_ranges = nullptr;
   long long* d_nodes = nullptr;
+  void* d_field = nullptr;  // olbm::FieldDesc of every domain (init, moments)
+  int field_blocks = 0;     // blocks of those kernels over all domains
   int ntiles = 0;
   // launch kind 2: the two-step tiles (2 NC - 2 columns) and their per-domain ranges;
   // the single steps of an odd count take the kind 1 tiles above
@@ -116,14 +118,21 @@ struct lbm_batch {
   bool initialised = false;
   int diag_every = 0;
   long long last_diag_t = -1;
-  cudaGraphExec_t graph = nullptr;
-  long long graph_key[4] = {-1, -1, -1, -1};
-  int graph_parity_end = 0;  // buffer holding the state after a replay of `graph`
+  // Graph of one call per buffer parity, so that calls that leave the state in the
+  // other buffer (an odd number of launches) do not capture again each time.
+  struct Replay {
+    cudaGraphExec_t exec = nullptr;
+    long long key[3] = {-1, -1, -1};
+    int parity_end = 0;  // buffer holding the state after a replay
+    void drop() {
+      if (exec) cudaGraphExecDestroy(exec);
+      exec = nullptr;
+    }
+  };
+  Replay graph[2];
   // Persistent mode: the barrier reset and the cooperative launch of n steps,
   // captured once per (n, buffer parity) and replayed.
-  cudaGraphExec_t pgraph = nullptr;
-  long long pgraph_key[2] = {-1, -1};
-  int pgraph_parity_end = 0;  // buffer holding the state after a replay of `pgraph`
+  Replay pgraph[2];
   char err[320] = {0};
 };
 
@@ -232,21 +241,13 @@ int build_tiles(lbm_batch* b) {
   if (e == cudaSuccess && !tiles2.empty())
     e = cudaMemcpy(b->d_ranges2, ranges2.data(), sizeof(int2) * ranges2.size(), cudaMemcpyHostToDevice);
   if (e != cudaSuccess) return bcuda(b, e, "lbm_batch tile upload");
-  if (b->graph) {
-    cudaGraphExecDestroy(b->graph);
-    b->graph = nullptr;
-  }
-  if (b->pgraph) {
-    cudaGraphExecDestroy(b->pgraph);
-    b->pgraph = nullptr;
-  }
+  for (int q = 0; q < 2; ++q) b->graph[q].drop(), b->pgraph[q].drop();
   return LBM_OK;
 }
 
 void free_batch(lbm_batch* b) {
   if (!b) return;
-  if (b->graph) cudaGraphExecDestroy(b->graph);
-  if (b->pgraph) cudaGraphExecDestroy(b->pgraph);
+  for (int q = 0; q < 2; ++q) b->graph[q].drop(), b->pgraph[q].drop();
   if (b->capture) cudaStreamDestroy(b->capture);
   if (b->capture_side) cudaStreamDestroy(b->capture_side);
   for (int k = 0; k < lbm_batch::kParts; ++k) {
@@ -261,6 +262,7 @@ void free_batch(lbm_batch* b) {
   cudaFree(b->d_tiles2);
   cudaFree(b->d_ranges2);
   cudaFree(b->d_nodes);
+  cudaFree(b->d_field);
   cudaFree(b->d_diag);
   cudaFree(b->d_diag_now);
   cudaFree(b->d_sticky);
@@ -420,6 +422,7 @@ int lbm_batch_create(int n, const int* nx, const int* ny, const double* theta, c
       (size_t)n * (prec == LBM_F64 ? sizeof(olbm::Desc<double>) : sizeof(olbm::Desc<float>));
   if ((e = cudaMalloc(&b->arena, arena)) != cudaSuccess || (e = cudaMalloc(&b->d_desc, desc_bytes)) != cudaSuccess ||
       (e = cudaMalloc(&b->d_nodes, sizeof(long long) * n)) != cudaSuccess ||
+      (e = cudaMalloc(&b->d_field, sizeof(olbm::FieldDesc) * n)) != cudaSuccess ||
       (e = cudaMalloc(&b->d_diag, sizeof(double) * 5 * n)) != cudaSuccess ||
       (e = cudaMalloc(&b->d_diag_now, sizeof(double) * 5 * n)) != cudaSuccess ||
       (e = cudaMalloc(&b->d_sticky, sizeof(unsigned long long))) != cudaSuccess ||
@@ -439,6 +442,25 @@ int lbm_batch_create(int n, const int* nx, const int* ny, const double* theta, c
     fill_desc(b, d);
     e = cudaMemcpy(b->d_desc, d.data(), desc_bytes, cudaMemcpyHostToDevice);
   }
+  std::vector<olbm::FieldDesc> field(n);
+  long long blocks = 0;
+  for (int k = 0; k < n; ++k) {
+    olbm::FieldDesc& d = field[k];
+    d = olbm::field_desc(b->geo[k], theta[k]);
+    d.node0 = b->node0[k];
+    long long bytes = 0;
+    lbm_layout(nx[k], ny[k], prec, nullptr, nullptr, &bytes);
+    d.buf[0] = b->arena + b->off[k];
+    d.buf[1] = b->arena + b->off[k] + (size_t)bytes;
+    d.blk0 = (int)blocks;
+    blocks += olbm::node_blocks(b->geo[k]);
+    if (blocks > 0x7fffffff) {
+      free_batch(b);
+      return bfail(nullptr, LBM_EINVAL, "lbm_batch_create: too many nodes");
+    }
+  }
+  b->field_blocks = (int)blocks;
+  if (e == cudaSuccess) e = cudaMemcpy(b->d_field, field.data(), sizeof(olbm::FieldDesc) * n, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(b->d_nodes, nodes.data(), sizeof(long long) * n, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemset(b->arena, 0, arena);
   if (e == cudaSuccess) e = cudaMemset(b->d_sticky, 0, sizeof(unsigned long long));
@@ -547,20 +569,16 @@ int lbm_batch_init(lbm_batch* b, const double* d_rho, const double* d_ux, const 
   int s = check_batch(b);
   if (s != LBM_OK) return s;
   if (!d_rho || !d_ux || !d_uy) return bfail(b, LBM_EINVAL, "lbm_batch_init: NULL field pointer");
-  for (int k = 0; k < b->n; ++k) {
-    long long bytes = 0;
-    lbm_layout(b->geo[k].nx, b->geo[k].ny, b->prec, nullptr, nullptr, &bytes);
-    void* dst = b->arena + b->off[k] + (size_t)(b->cur ? bytes : 0);
-    const long long o = b->node0[k];
-    cudaError_t e;
-    switch (b->prec) {
-      case LBM_F64: e = olbm::launch_init_f64(d_rho + o, d_ux + o, d_uy + o, b->geo[k], b->theta[k], b->rho_ref, dst, b->stream); break;
-      case LBM_F32_SHIFT: e = olbm::launch_init_f32(d_rho + o, d_ux + o, d_uy + o, b->geo[k], b->theta[k], b->rho_ref, dst, b->stream); break;
-      default: e = olbm::launch_init_f16(d_rho + o, d_ux + o, d_uy + o, b->geo[k], b->theta[k], b->rho_ref, dst, b->stream); break;
-    }
-    if (e != cudaSuccess) return bcuda(b, e, "lbm_batch_init");
+  // one launch for all domains (256 launches of small grids took 4.5 ms over 24 M nodes)
+  cudaError_t e;
+  const auto* desc = static_cast<const olbm::FieldDesc*>(b->d_field);
+  switch (b->prec) {
+    case LBM_F64: e = olbm::batch_init_f64(d_rho, d_ux, d_uy, desc, b->n, b->field_blocks, b->cur, b->rho_ref, b->stream); break;
+    case LBM_F32_SHIFT: e = olbm::batch_init_f32(d_rho, d_ux, d_uy, desc, b->n, b->field_blocks, b->cur, b->rho_ref, b->stream); break;
+    default: e = olbm::batch_init_f16(d_rho, d_ux, d_uy, desc, b->n, b->field_blocks, b->cur, b->rho_ref, b->stream); break;
   }
-  cudaError_t e = cudaMemsetAsync(b->d_sticky, 0, sizeof(unsigned long long), b->stream);
+  if (e != cudaSuccess) return bcuda(b, e, "lbm_batch_init");
+  e = cudaMemsetAsync(b->d_sticky, 0, sizeof(unsigned long long), b->stream);
   if (e != cudaSuccess) return bcuda(b, e, "lbm_batch_init reset");
   b->initialised = true;
   b->t = 0;
@@ -608,18 +626,14 @@ int lbm_batch_moments(lbm_batch* b, double* d_rho, double* d_ux, double* d_uy) {
   int s = check_batch(b);
   if (s != LBM_OK) return s;
   if (!d_rho || !d_ux || !d_uy) return bfail(b, LBM_EINVAL, "lbm_batch_moments: NULL field pointer");
-  for (int k = 0; k < b->n; ++k) {
-    const void* src = domain_buffer(b, k, b->cur);
-    const long long o = b->node0[k];
-    cudaError_t e;
-    switch (b->prec) {
-      case LBM_F64: e = olbm::launch_moments_f64(src, b->geo[k], b->rho_ref, d_rho + o, d_ux + o, d_uy + o, b->stream); break;
-      case LBM_F32_SHIFT: e = olbm::launch_moments_f32(src, b->geo[k], b->rho_ref, d_rho + o, d_ux + o, d_uy + o, b->stream); break;
-      default: e = olbm::launch_moments_f16(src, b->geo[k], b->rho_ref, d_rho + o, d_ux + o, d_uy + o, b->stream); break;
-    }
-    if (e != cudaSuccess) return bcuda(b, e, "lbm_batch_moments");
+  cudaError_t e;
+  const auto* desc = static_cast<const olbm::FieldDesc*>(b->d_field);
+  switch (b->prec) {
+    case LBM_F64: e = olbm::batch_moments_f64(desc, b->n, b->field_blocks, b->cur, b->rho_ref, d_rho, d_ux, d_uy, b->stream); break;
+    case LBM_F32_SHIFT: e = olbm::batch_moments_f32(desc, b->n, b->field_blocks, b->cur, b->rho_ref, d_rho, d_ux, d_uy, b->stream); break;
+    default: e = olbm::batch_moments_f16(desc, b->n, b->field_blocks, b->cur, b->rho_ref, d_rho, d_ux, d_uy, b->stream); break;
   }
-  return LBM_OK;
+  return e == cudaSuccess ? LBM_OK : bcuda(b, e, "lbm_batch_moments");
 }
 
 int lbm_batch_step(lbm_batch* b, int n) {
@@ -633,12 +647,9 @@ int lbm_batch_step(lbm_batch* b, int n) {
   if (b->mode == LBM_BATCH_PERSISTENT) {
     // One persistent cooperative launch for the n steps, captured with its barrier
     // reset into a CUDA graph once per (n, buffer parity) and replayed.
-    const long long pkey[2] = {n, b->cur};
-    if (!b->pgraph || !std::equal(pkey, pkey + 2, b->pgraph_key)) {
-      if (b->pgraph) {
-        cudaGraphExecDestroy(b->pgraph);
-        b->pgraph = nullptr;
-      }
+    lbm_batch::Replay& r = b->pgraph[b->cur];
+    if (!r.exec || r.key[0] != n) {
+      r.drop();
       cudaGraph_t g = nullptr;
       e = cudaStreamBeginCapture(b->capture, cudaStreamCaptureModeThreadLocal);
       if (e != cudaSuccess) return bcuda(b, e, "lbm_batch_step persistent capture");
@@ -646,40 +657,38 @@ int lbm_batch_step(lbm_batch* b, int n) {
       const cudaError_t le = b->cfg.kind == 2 && n >= 2
                                  ? launch_persistent_pairs(b, n, b->cur, b->capture, parity_end)
                                  : launch_persistent(b, n, b->cur, b->capture);
-      b->pgraph_parity_end = parity_end;
+      r.parity_end = parity_end;
       e = cudaStreamEndCapture(b->capture, &g);
       if (le != cudaSuccess || e != cudaSuccess) {
         if (g) cudaGraphDestroy(g);
         cudaGetLastError();
         return bcuda(b, le != cudaSuccess ? le : e, "lbm_batch_step persistent capture");
       }
-      e = cudaGraphInstantiate(&b->pgraph, g, 0);
+      e = cudaGraphInstantiate(&r.exec, g, 0);
       cudaGraphDestroy(g);
       if (e != cudaSuccess) {
-        b->pgraph = nullptr;
+        r.exec = nullptr;
         return bcuda(b, e, "lbm_batch_step persistent graph instantiate");
       }
-      std::copy(pkey, pkey + 2, b->pgraph_key);
+      r.key[0] = n;
     }
-    e = cudaGraphLaunch(b->pgraph, b->stream);
+    e = cudaGraphLaunch(r.exec, b->stream);
     if (e != cudaSuccess) return bcuda(b, e, "lbm_batch_step persistent launch");
     int timed_out = 0;
     e = cudaMemcpyAsync(&timed_out, &b->d_bar->err, sizeof(int), cudaMemcpyDeviceToHost, b->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
     if (e != cudaSuccess) return bcuda(b, e, "lbm_batch_step persistent");
-    b->cur = b->pgraph_parity_end;
+    b->cur = r.parity_end;
     b->t += n;
     if (timed_out) return bfail(b, LBM_ETIMEOUT, "a grid barrier of the persistent batch kernel timed out");
     return LBM_OK;
   }
   // Graph mode: capture the n launches once per (n, parity, diagnostics phase), replay.
   const long long phase = b->diag_every > 0 ? b->t % b->diag_every : -1;
-  const long long key[4] = {n, b->cur, b->diag_every, phase};
-  if (!b->graph || !std::equal(key, key + 4, b->graph_key)) {
-    if (b->graph) {
-      cudaGraphExecDestroy(b->graph);
-      b->graph = nullptr;
-    }
+  const long long key[3] = {n, b->diag_every, phase};
+  lbm_batch::Replay& r = b->graph[b->cur];
+  if (!r.exec || !std::equal(key, key + 3, r.key)) {
+    r.drop();
     cudaGraph_t g = nullptr;
     e = cudaStreamBeginCapture(b->capture, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return bcuda(b, e, "lbm_batch_step capture");
@@ -727,29 +736,29 @@ int lbm_batch_step(lbm_batch* b, int n) {
       }
       parity ^= 1;
     }
-    b->graph_parity_end = parity;
+    r.parity_end = parity;
     if (le == cudaSuccess && last >= 0) le = cudaStreamWaitEvent(b->capture, b->ev_fin[last], 0);  // join
     e = cudaStreamEndCapture(b->capture, &g);
     if (le != cudaSuccess || e != cudaSuccess) {
       if (g) cudaGraphDestroy(g);
       return bcuda(b, le != cudaSuccess ? le : e, "lbm_batch_step capture");
     }
-    e = cudaGraphInstantiate(&b->graph, g, 0);
+    e = cudaGraphInstantiate(&r.exec, g, 0);
     cudaGraphDestroy(g);
     if (e != cudaSuccess) {
-      b->graph = nullptr;
+      r.exec = nullptr;
       return bcuda(b, e, "lbm_batch_step graph instantiate");
     }
-    std::copy(key, key + 4, b->graph_key);
+    std::copy(key, key + 3, r.key);
   }
-  e = cudaGraphLaunch(b->graph, b->stream);
+  e = cudaGraphLaunch(r.exec, b->stream);
   if (e != cudaSuccess) return bcuda(b, e, "lbm_batch_step graph launch");
   if (b->diag_every > 0) {
     const long long last = b->t + n - 1;
     const long long ld = last - (last % b->diag_every);  // latest fused pass in [t, t + n), if any
     if (ld >= b->t) b->last_diag_t = ld;
   }
-  b->cur = b->graph_parity_end;
+  b->cur = r.parity_end;
   b->t += n;
   return LBM_OK;
 }

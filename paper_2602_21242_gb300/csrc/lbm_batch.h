@@ -57,7 +57,11 @@ struct BatchLaunch {
   cudaError_t batch_prepare_##SUFFIX(const BatchLaunch& b);                                                 \
   cudaError_t batch_step_##SUFFIX(const BatchLaunch& b, bool diag, int parity, cudaStream_t st);           \
   cudaError_t batch_persistent_##SUFFIX(const BatchLaunch& b, int n, int parity0, cudaStream_t st);        \
-  cudaError_t batch_diag_##SUFFIX(const BatchLaunch& b, int parity, double rho_ref, cudaStream_t st);
+  cudaError_t batch_diag_##SUFFIX(const BatchLaunch& b, int parity, double rho_ref, cudaStream_t st);        \
+  cudaError_t batch_init_##SUFFIX(const double* rho, const double* ux, const double* uy, const FieldDesc* desc, \
+                                  int n, int blocks, int parity, double rho_ref, cudaStream_t st);          \
+  cudaError_t batch_moments_##SUFFIX(const FieldDesc* desc, int n, int blocks, int parity, double rho_ref,  \
+                                     double* rho, double* ux, double* uy, cudaStream_t st);
 
 OLBM_DECLARE_BATCH(f64)
 OLBM_DECLARE_BATCH(f32)

@@ -634,14 +634,9 @@ struct FixedMoments {
   long long rho, jx, jy, ke2;  // 60 fraction bits; ke2 = j.u, twice the kinetic energy
 };
 
-// Collision of one FP64 node in fixed point (lbm_fixed.cuh); false for a node outside its
-// range, for which nothing is stored: that is a property of the node alone. next(f) is called
-// as soon as f is free and may load the next node's populations into it; sink receives the
-// node's FixedMoments and store(i, v) each post-collision population.
-template <int MODEL, typename Sink, typename Next, typename Store>
-__device__ __forceinline__ bool collide_fixed(double (&f)[9], const fx::Coefs& c, Sink&& sink, Next&& next,
-                                              Store&& store) {
-  fx::Fx<60> a[9], o[9];
+// The nine populations of a node with 60 fraction bits; false unless each is below 1 in
+// magnitude (and finite).
+__device__ __forceinline__ bool to_fixed(const double (&f)[9], fx::Fx<60> (&a)[9]) {
   // sign and magnitude of all nine at once: +0 <= f_i < 1 is the common case
   unsigned top = 0;
 #pragma unroll
@@ -658,6 +653,18 @@ __device__ __forceinline__ bool collide_fixed(double (&f)[9], const fx::Coefs& c
       ok = ok && ((unsigned)__double2hiint(f[i]) & 0x7FFFFFFFu) < 0x3FF00000u;
     }
   }
+  return ok;
+}
+
+// Collision of one FP64 node in fixed point (lbm_fixed.cuh); false for a node outside its
+// range, for which nothing is stored: that is a property of the node alone. next(f) is called
+// as soon as f is free and may load the next node's populations into it; sink receives the
+// node's FixedMoments and store(i, v) each post-collision population.
+template <int MODEL, typename Sink, typename Next, typename Store>
+__device__ __forceinline__ bool collide_fixed(double (&f)[9], const fx::Coefs& c, Sink&& sink, Next&& next,
+                                              Store&& store) {
+  fx::Fx<60> a[9], o[9];
+  bool ok = to_fixed(f, a);
   next(f);
   const fx::Moments m = fx::moments(a);
   ok = ok && fx::moments_in_range(m.rho, m.jx, m.jy);

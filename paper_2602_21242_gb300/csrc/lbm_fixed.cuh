@@ -149,6 +149,7 @@ struct Coefs {
   FxOp<61> e2;         // (1 - theta) / (2 theta) (polynomial equilibrium)
   Fx<62> theta, h, t, c3;
   Fx<60> v0;           // (1 - theta) / theta
+  Fx<60> theta2;       // theta^2
   int on;              // theta in the range of the formats
 };
 
@@ -175,6 +176,7 @@ inline Coefs make_coefs(double theta, double tau) {
   c.t = fx_of<62>(th * (1.0L - 3.0L * th));
   c.c3 = fx_of<62>(1.0L - 3.0L * th);
   c.v0 = fx_of<60>((1.0L - th) / th);
+  c.theta2 = fx_of<60>(th * th);
   return c;
 }
 
@@ -189,18 +191,18 @@ OLBM_EMU_HD u64 shr64(u64 v, uint32_t s) {
 #endif
 }
 
-// |x| truncated to 60 fraction bits; zeros and subnormals give 0. |x| < 8.
-OLBM_EMU_HD Fx<60> magnitude(double x) {
+// |x| truncated to F fraction bits, |x| < 2^(63 - F); zeros and subnormals give 0.
+template <int F = 60> OLBM_EMU_HD Fx<F> magnitude(double x) {
   const u64 u = emu::bits_of(x);
   const uint32_t e = (uint32_t)(u >> 52) & 0x7FFu;
-  return Fx<60>{(i64)shr64((u << 11) | emu::kSign, 1026u - e)};
+  return Fx<F>{(i64)shr64((u << 11) | emu::kSign, (uint32_t)(1086 - F) - e)};
 }
 OLBM_EMU_HD Fx<60> nonnegative(double x) {  // x >= +0
   const u64 u = emu::bits_of(x);
   return Fx<60>{(i64)shr64((u << 11) | emu::kSign, 1026u - (uint32_t)(u >> 52))};
 }
-OLBM_EMU_HD Fx<60> any_sign(double x) {
-  const Fx<60> m = magnitude(x);
+template <int F = 60> OLBM_EMU_HD Fx<F> any_sign(double x) {
+  const Fx<F> m = magnitude<F>(x);
   return (emu::bits_of(x) & emu::kSign) ? -m : m;
 }
 
@@ -209,10 +211,10 @@ OLBM_EMU_HD Fx<60> any_sign(double x) {
 // with b in its low mantissa bits; a - 2^8 has at most 20 bits, so its FP32
 // conversion is exact and widens by moving its exponent field; one FP64 addition
 // rounds their sum once.
-template <int F> OLBM_EMU_HD double to_double(Fx<F> x) {
+OLBM_EMU_HD double to_double(i64 v, int F) {
 #if defined(__CUDA_ARCH__)
-  const int32_t vh = (int32_t)(x.v >> 32);
-  const uint32_t vl = (uint32_t)x.v;
+  const int32_t vh = (int32_t)(v >> 32);
+  const uint32_t vl = (uint32_t)v;
   const int32_t a = (vh >> 12) - 256;
   const int32_t fb = __float_as_int(__int2float_rn(a));
   const uint32_t hh = ((uint32_t)(fb >> 3) & 0x8FFFFFFFu) + ((uint32_t)(896 + 44 - F) << 20);
@@ -220,8 +222,30 @@ template <int F> OLBM_EMU_HD double to_double(Fx<F> x) {
   const double lo = __hiloint2double((int)(((uint32_t)vh & 0xFFFu) | ((uint32_t)(1075 - F) << 20)), (int)vl);
   return hi + lo;
 #else
-  return __builtin_ldexp((double)x.v, -F);
+  return __builtin_ldexp((double)v, -F);
 #endif
+}
+template <int F> OLBM_EMU_HD double to_double(Fx<F> x) { return to_double(x.v, F); }
+
+// v 2^-F rounded to FP32 (to nearest). safe is cleared where v lies within 2^-50 of the
+// midpoint of two FP32 numbers (or is so small that this cannot be told): there a
+// result computed with an error below 2^-50 may round the other way.
+template <int F> OLBM_EMU_HD float to_float(Fx<F> x, bool& safe) {
+  const bool neg = x.v < 0;
+  const u64 a = neg ? 0 - (u64)x.v : (u64)x.v;
+  const uint32_t ah = (uint32_t)(a >> 32);
+  const int t = 31 - emu::clz32(ah | 1u);  // top bit of the high word
+  const u64 m = a << (31 - t);             // leading bit at 63
+  const uint32_t mh = (uint32_t)(m >> 32), rem = ((mh & 0xFFu) << 8) | ((uint32_t)m >> 24);
+  const uint32_t off = rem - 0x8000u, dist = rem >= 0x8000u ? off : 0u - off;
+  safe = safe & (ah >> 1 != 0) & (dist > ((1u << (F - 43)) >> t) + 1u);
+  const uint32_t bits = ((uint32_t)(127 + t + 32 - F - 1) << 23) + (mh >> 8) + (rem >> 15);
+  union {
+    uint32_t u;
+    float f;
+  } r;
+  r.u = bits | (neg ? 0x80000000u : 0u);
+  return r.f;
 }
 
 // ---------------------------------------------------------------- 1 / rho
@@ -258,6 +282,42 @@ OLBM_EMU_HD Fx<62> reciprocal(Fx<60> rho) {
 }
 
 // ---------------------------------------------------------------- one node
+// Populations from the nine moments sum a^p b^q f_(a,b): out[0] as it is, out[1..4]
+// twice, out[5..8] four times the population (Fig. 1a order).
+struct MomentSet {
+  Fx<60> M00, M10, M01, M20, M02, M11, M21, M12, M22;
+};
+OLBM_EMU_HD void populations(const MomentSet& M, Fx<60> (&out)[9]) {
+  const Fx<60> a0 = M.M00 - M.M20, a1 = M.M01 - M.M21, a2 = M.M02 - M.M22;  // column a = 0: b moments
+  const Fx<60> p0 = M.M20 + M.M10, q0 = M.M20 - M.M10;                      // columns a = +1, -1, doubled
+  const Fx<60> p1 = M.M21 + M.M11, q1 = M.M21 - M.M11, p2 = M.M22 + M.M12, q2 = M.M22 - M.M12;
+  out[0] = a0 - a2;
+  out[2] = a2 + a1, out[4] = a2 - a1;
+  out[1] = p0 - p2, out[3] = q0 - q2;
+  out[5] = p2 + p1, out[8] = p2 - p1, out[6] = q2 + q1, out[7] = q2 - q1;
+}
+
+// The guided equilibrium (Eq. 10) of one node, less the rest state of unit density if
+// SHIFT: rho in (0, 4), |u| < 1/2; out scaled as by populations().
+template <bool SHIFT>
+OLBM_EMU_HD void equilibrium(Fx<60> rho, Fx<64> u, Fx<64> v, const Coefs& c, Fx<60> (&out)[9]) {
+  const FxOp<60> ro = op(rho);
+  const FxOp<64> ux = op(u), uy = op(v);
+  const Fx<60> jx = ro * ux, jy = ro * uy;
+  const auto jxo = op(jx);
+  const Fx<60> rt = op(to<61>(rho)) * c.theta_op;
+  const Fx<60> rsx = rt + jxo * ux, rsy = rt + op(jy) * uy;
+  MomentSet M;
+  M.M00 = rho, M.M10 = jx, M.M01 = jy, M.M20 = rsx, M.M02 = rsy, M.M11 = jxo * uy;
+  M.M21 = op(rsx) * uy, M.M12 = op(rsy) * ux;
+  M.M22 = to<60>(op(to<61>(rsx)) * op(c.theta + to<62>(square(uy))));
+  if constexpr (SHIFT) {  // the rest state's moments: 1, theta, theta, theta^2
+    const Fx<60> th = to<60>(c.theta);
+    M.M00 = M.M00 - Fx<60>{(i64)1 << 60}, M.M20 = M.M20 - th, M.M02 = M.M02 - th, M.M22 = M.M22 - c.theta2;
+  }
+  populations(M, out);
+}
+
 OLBM_EMU_HD bool within(i64 v, int32_t bound) {  // |v's high word| < bound (slightly inside)
   return (uint32_t)((int32_t)(v >> 32) + (bound - 1)) < (uint32_t)(2 * bound - 2);
 }
@@ -354,14 +414,7 @@ OLBM_EMU_HD bool collide(const Moments& m, const Fx<60> (&f)[9], const Coefs& c,
       M01 = M01 + uy * op(Ay);
     }
   }
-  // moments -> populations
-  const Fx<60> a0 = rho - M20, a1 = M01 - M21, a2 = M02 - M22;        // column a = 0: b moments
-  const Fx<60> p0 = M20 + M10, q0 = M20 - M10;                        // columns a = +1, -1, doubled
-  const Fx<60> p1 = M21 + M11, q1 = M21 - M11, p2 = M22 + M12, q2 = M22 - M12;
-  out[0] = a0 - a2;
-  out[2] = a2 + a1, out[4] = a2 - a1;
-  out[1] = p0 - p2, out[3] = q0 - q2;
-  out[5] = p2 + p1, out[8] = p2 - p1, out[6] = q2 + q1, out[7] = q2 - q1;
+  populations(MomentSet{rho, M10, M01, M20, M02, M11, M21, M12, M22}, out);
   if constexpr (MODEL == 0 || MODEL == 5) {
     // f* = f^eq + omega' (f - f^eq), in the scaling of out
     out[0] = out[0] + op(to<61>(f[0] - out[0])) * c.omp;

@@ -570,57 +570,116 @@ __device__ __forceinline__ void pulled_moments(const typename Form<PREC>::S* __r
   jy = d24 + (d57 + d68);
 }
 
+// One node's FP64 contributions to the diagnostics.
+template <int PREC>
+__device__ __forceinline__ void diag_node(const typename Form<PREC>::S* __restrict__ src, const Geometry& g, int x,
+                                          int y, double rho_ref, double (&acc)[kNDiag]) {
+  double m0, jx, jy;
+  pulled_moments<PREC>(src, g, x, y, m0, jx, jy);
+  if (finite_bits(m0)) {
+    acc[0] += m0;
+    acc[1] += jx;
+    acc[2] += jy;
+    acc[3] = fma(0.5 * fma(jx, jx, jy * jy), recip(rho_ref + m0), acc[3]);
+  } else {
+    acc[4] += 1.0;
+  }
+}
+
+// Block totals of the accumulators of a diagnostics pass (sums and the count of nodes whose
+// populations do not sum to a finite value) into p[0 .. 4].
+__device__ __forceinline__ void diag_store(double (&acc)[kNDiag], const FixedDiagAcc& facc, double* __restrict__ p) {
+#pragma unroll
+  for (int k = 0; k < 4; ++k) acc[k] += facc.s[k].value() * (k == 3 ? 0.5 : 1.0);
+  double tot[kNDiag];
+  block_sum<kNDiag, kNT>(acc, tot);
+  if (threadIdx.x == 0 && threadIdx.y == 0) {
+#pragma unroll
+    for (int k = 0; k < kNDiag; ++k) p[k] = tot[k];
+  }
+}
+
 // Pull only (no collision): FP64 moments of f(x, t), block partials as above;
 // each thread takes kDiagRows rows of its column, so the block reduction is paid
 // once per kDiagRows nodes. The kinetic energy uses the reciprocal of the
-// collision (a density outside [2^-126, 2^126) makes it non-finite).
+// collision (a density outside [2^-126, 2^126) makes it non-finite). FP64 storage: nodes
+// in the range of the fixed-point collision are summed exactly in integers, with j.u of
+// their energy in fixed point, which leaves the pass to memory instead of the FP64 pipe
+// (2048^2: 291 us with every node on the FP64 pipe).
 template <int PREC>
 __global__ void __launch_bounds__(kNT) diag_kernel(const typename Form<PREC>::S* __restrict__ src, Geometry g,
                                                    double rho_ref, double* __restrict__ partials) {
   const int x = blockIdx.x * kBX + threadIdx.x;
   const int y0 = blockIdx.y * kBY * kDiagRows + threadIdx.y;
   double acc[kNDiag] = {0.0, 0.0, 0.0, 0.0, 0.0};
+  FixedDiagAcc facc;
   if (x < g.nx) {
     for (int r = 0; r < kDiagRows; ++r) {
       const int y = y0 + r * kBY;
       if (y >= g.ny) break;
-      double m0, jx, jy;
-      pulled_moments<PREC>(src, g, x, y, m0, jx, jy);
-      if (finite_bits(m0)) {
-        acc[0] += m0;
-        acc[1] += jx;
-        acc[2] += jy;
-        acc[3] = fma(0.5 * fma(jx, jx, jy * jy), recip(rho_ref + m0), acc[3]);
-      } else {
-        acc[4] += 1.0;
+      if constexpr (PREC == 0) {
+        long long o[9];
+        pull_offsets(x, y, g, o);
+        double f[9];
+#pragma unroll
+        for (int i = 0; i < 9; ++i) f[i] = src[i * g.plane + o[i]];
+        fx::Fx<60> a[9];
+        bool ok = to_fixed(f, a);
+        const fx::Moments m = fx::moments(a);
+        ok = ok && fx::moments_in_range(m.rho, m.jx, m.jy);
+        if (ok) {
+          const auto ir = fx::op(fx::reciprocal(m.rho));
+          const auto ux = fx::op(fx::to<64>(fx::op(fx::to<62>(m.jx)) * ir)), uy = fx::op(fx::to<64>(fx::op(fx::to<62>(m.jy)) * ir));
+          const fx::Fx<60> ke2 = fx::op(m.jx) * ux + fx::op(m.jy) * uy;
+          facc.add(FixedMoments{m.rho.v, m.jx.v, m.jy.v, ke2.v});
+          continue;
+        }
       }
+      diag_node<PREC>(src, g, x, y, rho_ref, acc);
     }
   }
-  double tot[kNDiag];
-  block_sum<kNDiag, kNT>(acc, tot);
-  if (threadIdx.x == 0 && threadIdx.y == 0) {
-    double* p = partials + (long long)(blockIdx.y * gridDim.x + blockIdx.x) * kNDiag;
-#pragma unroll
-    for (int k = 0; k < kNDiag; ++k) p[k] = tot[k];
-  }
+  diag_store(acc, facc, partials + (long long)(blockIdx.y * gridDim.x + blockIdx.x) * kNDiag);
 }
 
 // ------------------------------------------------------------------ init, moments, state copies
+// What the field kernels (init, moments) need of one lattice, or of one domain of a batch.
+struct FieldDesc {
+  Geometry g;
+  double theta;
+  fx::Coefs c;
+  long long node0;  // offset of its fields in the packed arrays (batch)
+  void* buf[2];     // its population buffers (batch)
+  int blk0;         // its first block of kBX x kBY nodes (batch)
+  int pad;
+};
+inline FieldDesc field_desc(const Geometry& g, double theta) {
+  FieldDesc d = {};
+  d.g = g;
+  d.theta = theta;
+  d.c = fx::make_coefs(theta, 1.0);
+  return d;
+}
+// The domain of block b: the last one whose first block is at most b.
+__device__ __forceinline__ int domain_of(const FieldDesc* __restrict__ d, int n, int b) {
+  int lo = 0, hi = n - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (d[mid].blk0 <= b) lo = mid;
+    else hi = mid - 1;
+  }
+  return lo;
+}
+
 // B_i(x) = f^eq_i(rho0(x + c_i), u0(x + c_i)) - rest_i: the buffer whose pull is f^eq(rho0, u0).
 // Written as a push (each element once): node x forms its nine f^eq_i from one
-// set of per-axis factors and stores them at x - c_i.
+// set of per-axis factors and stores them at x - c_i. In FP64 arithmetic; out of line,
+// for the nodes that init_node leaves out.
 template <int PREC>
-__global__ void __launch_bounds__(kNT) init_kernel(const double* __restrict__ rho, const double* __restrict__ ux,
-                                                   const double* __restrict__ uy, Geometry g, double theta,
-                                                   double rho_ref, typename Form<PREC>::S* __restrict__ dst) {
+__device__ __noinline__ void init_node_float(double r, double u, double v, const Geometry& g, int x, int y,
+                                             double theta, double rho_ref, typename Form<PREC>::S* __restrict__ dst) {
   using S = typename Form<PREC>::S;
-  const int x = blockIdx.x * kBX + threadIdx.x;
-  const int y = blockIdx.y * kBY + threadIdx.y;
-  if (x >= g.nx || y >= g.ny) return;
   long long o[9];
   pull_offsets(x, y, g, o);
-  const long long n = (long long)y * g.nx + x;
-  const double r = rho[n], u = ux[n], v = uy[n];
   const double px[3] = {geq_factor(-1, u, theta), geq_factor(0, u, theta), geq_factor(1, u, theta)};
   const double py[3] = {geq_factor(-1, v, theta), geq_factor(0, v, theta), geq_factor(1, v, theta)};
   const double rpx[3] = {r * px[0], r * px[1], r * px[2]};
@@ -634,7 +693,139 @@ __global__ void __launch_bounds__(kNT) init_kernel(const double* __restrict__ rh
   }
 }
 
+// The same in fixed point (lbm_fixed.cuh) for densities below 4 (shifted forms: 2) and
+// velocities below 1/2. FP64 arithmetic held this kernel on the FP64 pipe (33 operations a
+// node with the conversions to FP32: 1013 us in FP64 and 1279 us in FP32 at 4096^2 for
+// 96 and 60 bytes a node). The shifted forms store what the FP64 arithmetic stores, bit for
+// bit: a deviation within 2^-50 of a rounding boundary, more than either path's error
+// (at most 4 roundings of values below 2, and a few units of 2^-60), is left to it.
+template <int PREC>
+__device__ __forceinline__ void init_node(double r, double u, double v, const FieldDesc& d, int x, int y,
+                                          double rho_ref, typename Form<PREC>::S* __restrict__ dst) {
+  constexpr bool kShift = PREC != 0;
+  const unsigned rh = (unsigned)__double2hiint(r);
+  const unsigned uh = (unsigned)__double2hiint(u) & 0x7FFFFFFFu, vh = (unsigned)__double2hiint(v) & 0x7FFFFFFFu;
+  bool ok = d.c.on && rh < (kShift ? 0x40000000u : 0x40100000u) && uh < 0x3FE00000u && vh < 0x3FE00000u;
+  fx::Fx<60> f[9];
+  float s[9];
+  if (ok) {
+    fx::equilibrium<kShift>(fx::nonnegative(r), fx::any_sign<64>(u), fx::any_sign<64>(v), d.c, f);
+    if constexpr (kShift) {
+      s[0] = fx::to_float(f[0], ok);
+#pragma unroll
+      for (int i = 1; i < 5; ++i) s[i] = fx::to_float(fx::Fx<61>{f[i].v}, ok);
+#pragma unroll
+      for (int i = 5; i < 9; ++i) s[i] = fx::to_float(fx::Fx<62>{f[i].v}, ok);
+    }
+  }
+  if (!ok) {
+    init_node_float<PREC>(r, u, v, d.g, x, y, d.theta, rho_ref, dst);
+    return;
+  }
+  long long o[9];
+  pull_offsets(x, y, d.g, o);
+#pragma unroll
+  for (int i = 0; i < 9; ++i) {
+    auto* q = dst + i * d.g.plane + o[i];
+    if constexpr (kShift) st_t(q, s[i]);
+    else *q = fx::to_double(f[i].v, i == 0 ? 60 : (i < 5 ? 61 : 62));
+  }
+}
+
+template <int PREC>
+__global__ void __launch_bounds__(kNT) init_kernel(const double* __restrict__ rho, const double* __restrict__ ux,
+                                                   const double* __restrict__ uy, FieldDesc d, double rho_ref,
+                                                   typename Form<PREC>::S* __restrict__ dst) {
+  const int x = blockIdx.x * kBX + threadIdx.x;
+  const int y = blockIdx.y * kBY + threadIdx.y;
+  if (x >= d.g.nx || y >= d.g.ny) return;
+  const long long n = (long long)y * d.g.nx + x;
+  init_node<PREC>(rho[n], ux[n], uy[n], d, x, y, rho_ref, dst);
+}
+
+// Every domain of a batch in one launch: block b is a block of kBX x kBY nodes of one domain.
+template <int PREC>
+__global__ void __launch_bounds__(kNT) batch_init_kernel(const double* __restrict__ rho, const double* __restrict__ ux,
+                                                         const double* __restrict__ uy,
+                                                         const FieldDesc* __restrict__ desc, int ndom, int parity,
+                                                         double rho_ref) {
+  const FieldDesc& d = desc[domain_of(desc, ndom, blockIdx.x)];
+  const int b = blockIdx.x - d.blk0, strips = (d.g.nx + kBX - 1) / kBX;
+  const int x = b % strips * kBX + threadIdx.x, y = b / strips * kBY + threadIdx.y;
+  if (x >= d.g.nx || y >= d.g.ny) return;
+  const long long n = d.node0 + (long long)y * d.g.nx + x;
+  init_node<PREC>(rho[n], ux[n], uy[n], d, x, y, rho_ref, static_cast<typename Form<PREC>::S*>(d.buf[parity]));
+}
+
+// FP64 sums of the pulled populations of one node, out of line (the nodes that
+// pulled_sums leaves out).
+template <int PREC>
+__device__ __noinline__ void pulled_moments_cold(const typename Form<PREC>::S* __restrict__ src, const Geometry& g,
+                                                 int x, int y, double* m0, double* jx, double* jy) {
+  pulled_moments<PREC>(src, g, x, y, *m0, *jx, *jy);
+}
+
+// The sums m0, j_x, j_y of node (x, y)'s stored values, rounded to binary64, added as
+// 64-bit integers: FP64 storage with 60 fraction bits (populations below 1), the shifted
+// forms with the largest of the nine at bit 58, so that values down to 2^-35 of it are
+// exact. Left to FP64 arithmetic, the 16 additions (and nine conversions from FP32) held
+// this kernel on the FP64 pipe.
+template <int PREC>
+__device__ __forceinline__ void pulled_sums(const typename Form<PREC>::S* __restrict__ src, const Geometry& g, int x,
+                                            int y, double& m0, double& jx, double& jy) {
+  long long o[9];
+  pull_offsets(x, y, g, o);
+  fx::Fx<60> a[9];
+  int F = 60;
+  bool ok;
+  if constexpr (PREC == 0) {
+    double f[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) f[i] = src[i * g.plane + o[i]];
+    ok = to_fixed(f, a);
+  } else {
+    float f[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) f[i] = ld_t(src + i * g.plane + o[i], 0.0f);
+    int top = 1;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) top = max(top, (__float_as_int(f[i]) & 0x7FFFFFFF) >> 23);
+    ok = top > 32 && top < 160;  // the exponent arithmetic below stays in range
+    F = 185 - top;               // value = integer 2^-F
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+      const unsigned b = __float_as_uint(f[i]), e = (b >> 23) & 0xFFu;
+      const unsigned man = (b & 0x7FFFFFu) | (e != 0 ? 0x800000u : 0u);
+      const long long v = (long long)fx::shr64((unsigned long long)man << 35, (unsigned)top - max(e, 1u));
+      a[i] = fx::Fx<60>{(int)b < 0 ? -v : v};
+    }
+  }
+  const fx::Moments m = fx::moments(a);
+  if constexpr (PREC == 0) {  // (sums below 4 for the conversion)
+    ok = ok && fx::within(m.rho.v, 1 << 30) && fx::within(m.jx.v, 1 << 30) && fx::within(m.jy.v, 1 << 30);
+  }
+  if (!ok) {
+    pulled_moments_cold<PREC>(src, g, x, y, &m0, &jx, &jy);
+    return;
+  }
+  m0 = fx::to_double(m.rho.v, F), jx = fx::to_double(m.jx.v, F), jy = fx::to_double(m.jy.v, F);
+}
+
 // (rho, u) of f(x, t) in FP64, unpadded [y][x] output.
+template <int PREC>
+__device__ __forceinline__ void moments_node(const typename Form<PREC>::S* __restrict__ src, const Geometry& g, int x,
+                                             int y, double rho_ref, double* __restrict__ rho, double* __restrict__ ux,
+                                             double* __restrict__ uy) {
+  double m0, jx, jy;
+  pulled_sums<PREC>(src, g, x, y, m0, jx, jy);
+  const double r = PREC == 0 ? m0 : rho_ref + m0;
+  const double ir = recip(r);  // a density outside [2^-126, 2^126) gives non-finite velocities
+  const long long n = (long long)y * g.nx + x;
+  rho[n] = r;
+  ux[n] = jx * ir;
+  uy[n] = jy * ir;
+}
+
 template <int PREC>
 __global__ void __launch_bounds__(kNT) moments_kernel(const typename Form<PREC>::S* __restrict__ src, Geometry g,
                                                       double rho_ref, double* __restrict__ rho,
@@ -642,14 +833,20 @@ __global__ void __launch_bounds__(kNT) moments_kernel(const typename Form<PREC>:
   const int x = blockIdx.x * kBX + threadIdx.x;
   const int y = blockIdx.y * kBY + threadIdx.y;
   if (x >= g.nx || y >= g.ny) return;
-  double m0, jx, jy;
-  pulled_moments<PREC>(src, g, x, y, m0, jx, jy);
-  const double r = rho_ref + m0;
-  const double ir = recip(r);  // a density outside [2^-126, 2^126) gives non-finite velocities
-  const long long n = (long long)y * g.nx + x;
-  rho[n] = r;
-  ux[n] = jx * ir;
-  uy[n] = jy * ir;
+  moments_node<PREC>(src, g, x, y, rho_ref, rho, ux, uy);
+}
+
+// Every domain of a batch in one launch.
+template <int PREC>
+__global__ void __launch_bounds__(kNT) batch_moments_kernel(const FieldDesc* __restrict__ desc, int ndom, int parity,
+                                                            double rho_ref, double* __restrict__ rho,
+                                                            double* __restrict__ ux, double* __restrict__ uy) {
+  const FieldDesc& d = desc[domain_of(desc, ndom, blockIdx.x)];
+  const int b = blockIdx.x - d.blk0, strips = (d.g.nx + kBX - 1) / kBX;
+  const int x = b % strips * kBX + threadIdx.x, y = b / strips * kBY + threadIdx.y;
+  if (x >= d.g.nx || y >= d.g.ny) return;
+  moments_node<PREC>(static_cast<const typename Form<PREC>::S*>(d.buf[parity]), d.g, x, y, rho_ref, rho + d.node0,
+                     ux + d.node0, uy + d.node0);
 }
 
 // out_i(x) = B_i(x - c_i) + rest_i  (pre-collision f(x, t), FP64, unpadded [i][y][x]).
@@ -859,13 +1056,25 @@ template <int PREC> struct Launch {
 
   static cudaError_t init(const double* rho, const double* ux, const double* uy, const Geometry& g, double theta,
                           double rho_ref, void* dst, cudaStream_t st) {
-    init_kernel<PREC><<<grid_of(g), dim3(kBX, kBY), 0, st>>>(rho, ux, uy, g, theta, rho_ref, (S*)dst);
+    init_kernel<PREC><<<grid_of(g), dim3(kBX, kBY), 0, st>>>(rho, ux, uy, field_desc(g, theta), rho_ref, (S*)dst);
     return cudaGetLastError();
   }
 
   static cudaError_t moments(const void* src, const Geometry& g, double rho_ref, double* rho, double* ux,
                              double* uy, cudaStream_t st) {
     moments_kernel<PREC><<<grid_of(g), dim3(kBX, kBY), 0, st>>>((const S*)src, g, rho_ref, rho, ux, uy);
+    return cudaGetLastError();
+  }
+
+  static cudaError_t batch_init(const double* rho, const double* ux, const double* uy, const FieldDesc* desc, int n,
+                                int blocks, int parity, double rho_ref, cudaStream_t st) {
+    batch_init_kernel<PREC><<<blocks, dim3(kBX, kBY), 0, st>>>(rho, ux, uy, desc, n, parity, rho_ref);
+    return cudaGetLastError();
+  }
+
+  static cudaError_t batch_moments(const FieldDesc* desc, int n, int blocks, int parity, double rho_ref, double* rho,
+                                   double* ux, double* uy, cudaStream_t st) {
+    batch_moments_kernel<PREC><<<blocks, dim3(kBX, kBY), 0, st>>>(desc, n, parity, rho_ref, rho, ux, uy);
     return cudaGetLastError();
   }
 
@@ -899,6 +1108,14 @@ template <int PREC> struct Launch {
   cudaError_t launch_moments_##SUFFIX(const void* src, const Geometry& g, double rho_ref, double* rho,           \
                                       double* ux, double* uy, cudaStream_t st) {                                 \
     return Launch<PREC>::moments(src, g, rho_ref, rho, ux, uy, st);                                              \
+  }                                                                                                              \
+  cudaError_t batch_init_##SUFFIX(const double* rho, const double* ux, const double* uy, const FieldDesc* desc,  \
+                                  int n, int blocks, int parity, double rho_ref, cudaStream_t st) {              \
+    return Launch<PREC>::batch_init(rho, ux, uy, desc, n, blocks, parity, rho_ref, st);                          \
+  }                                                                                                              \
+  cudaError_t batch_moments_##SUFFIX(const FieldDesc* desc, int n, int blocks, int parity, double rho_ref,       \
+                                     double* rho, double* ux, double* uy, cudaStream_t st) {                     \
+    return Launch<PREC>::batch_moments(desc, n, blocks, parity, rho_ref, rho, ux, uy, st);                       \
   }                                                                                                              \
   cudaError_t launch_get_state_##SUFFIX(const void* src, const Geometry& g, double theta, double rho_ref,        \
                                         double* out, cudaStream_t st) {                                          \
