@@ -83,7 +83,9 @@ class Batch:
     def _packed(self, fields):
         out = []
         for name, parts in zip(("rho", "ux", "uy"), fields):
-            flat = torch.cat([torch.as_tensor(p, dtype=torch.float64).reshape(-1) for p in parts])
+            parts = [p if isinstance(p, torch.Tensor) and p.dtype == torch.float64
+                     else torch.as_tensor(p, dtype=torch.float64) for p in parts]
+            flat = torch.cat([p.reshape(-1) for p in parts])
             if flat.numel() != self.total_nodes:
                 raise ValueError(f"{name}: expected {self.total_nodes} values")
             out.append(flat.to(self.device).contiguous())
@@ -126,11 +128,8 @@ class Batch:
         with torch.cuda.device(self.device):
             capi.lbm_batch_moments(self._b, out[0].data_ptr(), out[1].data_ptr(), out[2].data_ptr())
             self.stream.synchronize()
-        res = []
-        for k in range(self.n):
-            a, b = int(self.offsets[k]), int(self.offsets[k + 1])
-            res.append(tuple(out[j, a:b].reshape(self.ny[k], self.nx[k]) for j in range(3)))
-        return res
+        # two views a domain and one split, not six (256 domains: 4.6 ms of host time before)
+        return [d.view(3, ny, nx).unbind(0) for d, ny, nx in zip(out.split(self.sizes, dim=1), self.ny, self.nx)]
 
     def diagnostics(self, raise_nonfinite: bool = True):
         with torch.cuda.device(self.device):
