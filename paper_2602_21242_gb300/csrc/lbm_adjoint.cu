@@ -14,6 +14,7 @@
 #include "lbm.h"
 #include "lbm_adjoint.cuh"
 #include "lbm_ctx.h"
+#include "lbm_fixed_adjoint.cuh"
 #include "lbm_kernels.cuh"
 #include "lbm_walls.h"
 
@@ -76,21 +77,7 @@ __device__ __forceinline__ void adj_step_body(const typename Form<PREC>::S* __re
   };
   T f[9], mu[9], out[9];
   load(f, mu);
-  if constexpr (std::is_same<T, double>::value && OLBM_F64_EMU_MUL) {
-    // FP64: the products on the integer pipes, each with its own fallback to the
-    // FP64 instruction. (Without the fallbacks, checking the nine results once and
-    // redoing a node measured 1.4 % faster on the 1024^2 gradient, but a field that
-    // is zero over a region would redo every node there: one node a thread gives
-    // no later rows to switch to FP64 products for.)
-    d64c fe[9], me[9], oe[9];
-#pragma unroll
-    for (int i = 0; i < 9; ++i) fe[i] = d64c(f[i]), me[i] = d64c(mu[i]);
-    collide_vjp<MODEL, Form<PREC>::kShift, d64c>(fe, me, coef_cast<d64c>(c), oe);
-#pragma unroll
-    for (int i = 0; i < 9; ++i) out[i] = oe[i].v;
-  } else {
-    collide_vjp<MODEL, Form<PREC>::kShift, T>(f, mu, c, out);
-  }
+  collide_vjp<MODEL, Form<PREC>::kShift, T>(f, mu, c, out);
   const long long here = (long long)y * g.pitch + x;
 #pragma unroll
   for (int i = 0; i < 9; ++i) lam[i * g.plane + here] = out[i];
@@ -104,17 +91,88 @@ __global__ void __launch_bounds__(kABX* kABY) adj_step_kernel(const typename For
   adj_step_body<MODEL, PREC>(fbuf, lam_next, lam, g, c);
 }
 
-// The FP64 form, compiled for two blocks a SM (118 registers; with one it takes
-// 174 and the 1024^2 FP64 gradient's backward pass took 320 ms instead of 292).
+// f pulled at (x, y), and mu_i = lambda_i(t + 1) at x + c_i (the offset that pulls the
+// opposite population), periodic.
+__device__ __forceinline__ void adj_load_f64(const double* __restrict__ fbuf, const double* __restrict__ lam_next,
+                                             const Geometry& g, int x, int y, double (&f)[9], double (&mu)[9]) {
+  long long o[9];
+  pull_offsets(x, y, g, o);
+#pragma unroll
+  for (int i = 0; i < 9; ++i) f[i] = ld_plain(fbuf + i * g.plane + o[i]);
+#pragma unroll
+  for (int i = 0; i < 9; ++i)
+    mu[i] = ld_plain(lam_next + i * g.plane + o[i == 0 ? 0 : (i < 5 ? (i + 1) % 4 + 1 : (i - 3) % 4 + 5)]);
+}
+
+// One FP64 node in floating point, its products on the integer pipes, each with its own
+// fallback to the FP64 instruction; out of line, for the nodes that the fixed-point
+// derivative leaves out.
+template <int MODEL>
+__device__ __noinline__ void adj_node_float(const double* __restrict__ fbuf, const double* __restrict__ lam_next,
+                                            double* __restrict__ lam, const Geometry& g, const Coef<double>& c, int x,
+                                            int y) {
+  double f[9], mu[9];
+  adj_load_f64(fbuf, lam_next, g, x, y, f, mu);
+  d64c fe[9], me[9], oe[9];
+#pragma unroll
+  for (int i = 0; i < 9; ++i) fe[i] = d64c(f[i]), me[i] = d64c(mu[i]);
+  collide_vjp<MODEL, false, d64c>(fe, me, coef_cast<d64c>(c), oe);
+  double* out = lam + (long long)y * g.pitch + x;
+#pragma unroll
+  for (int i = 0; i < 9; ++i) out[i * g.plane] = oe[i].v;
+}
+
+// The FP64 form: the derivative in 64-bit fixed point (lbm_fixed_adjoint.cuh), one node a
+// thread, launched with programmatic serialization (plain loads after its wait). Bound by
+// the FP64 pipe before (about 210 of its operations a node, 82 % busy: 384^2 70 us a step),
+// now by the integer pipes (1024^2 gradient of 100 steps 14.2 ms with five blocks a SM, 14.5
+// with four, 14.9 with three; 384^2 12.2 -> 3.2 ms with the forward steps).
+constexpr int kAFX = 64, kAFY = 2;
 #ifndef OLBM_ADJ_F64_MINB
-#define OLBM_ADJ_F64_MINB 2
+#define OLBM_ADJ_F64_MINB 5
 #endif
 template <int MODEL>
-__global__ void __launch_bounds__(kABX* kABY, OLBM_ADJ_F64_MINB) adj_step_f64_kernel(const double* __restrict__ fbuf,
+__global__ void __launch_bounds__(kAFX* kAFY, OLBM_ADJ_F64_MINB) adj_step_f64_kernel(const double* __restrict__ fbuf,
                                                                                      const double* __restrict__ lam_next,
                                                                                      double* __restrict__ lam, Geometry g,
                                                                                      Coef<double> c) {
-  adj_step_body<MODEL, 0>(fbuf, lam_next, lam, g, c);
+  const int x = blockIdx.x * kAFX + threadIdx.x, y = blockIdx.y * kAFY + threadIdx.y;
+  pdl_wait();
+  pdl_launch_dependents();
+  if (x >= g.nx || y >= g.ny) return;
+  double f[9], mu[9];
+  adj_load_f64(fbuf, lam_next, g, x, y, f, mu);
+  bool ok = c.fixed.on != 0, zero = false;
+  int top = 0;
+  fx::Fx<60> l[9];
+  if (ok) {
+    fx::Fx<60> a[9], m[9];
+    ok = to_fixed(f, a);
+    const fx::Moments mo = fx::moments(a);
+    ok = ok && fx::moments_in_range(mo.rho, mo.jx, mo.jy);
+    // mu aligned to the largest of the nine: |mu| 2^(1018 - top) < 2^-4
+#pragma unroll
+    for (int i = 0; i < 9; ++i) top = max(top, (__double2hiint(mu[i]) >> 20) & 0x7FF);
+    unsigned long long any = 0;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+      const unsigned long long u = (unsigned long long)__double_as_longlong(mu[i]);
+      any |= u << 1;
+      const long long v = (long long)fx::shr64((u << 11) | emu::kSign, (unsigned)(8 + top) - ((unsigned)(u >> 52) & 0x7FFu));
+      m[i] = fx::Fx<60>{(long long)u < 0 ? -v : v};
+    }
+    zero = ok && any == 0;  // no cotangent reaches the node
+    ok = ok && top > 200 && top < 1900;
+    ok = ok && fx::collide_vjp<MODEL>(mo, m, c.fixed, l);
+  }
+  double* out = lam + (long long)y * g.pitch + x;
+  if (__any_sync(__activemask(), !ok && !zero)) {
+    if (!ok && !zero) adj_node_float<MODEL>(fbuf, lam_next, lam, g, c, x, y);
+  }
+  if (ok || zero) {
+#pragma unroll
+    for (int i = 0; i < 9; ++i) out[i * g.plane] = zero ? 0.0 : fx::to_double(l[i].v, 1078 - top);
+  }
 }
 
 // The FP32 form on node pairs (x, x + 1), x even, with packed f32x2 arithmetic
@@ -207,8 +265,9 @@ template <int PREC> struct Adjoint {
       }
     }
     if constexpr (PREC == 0) {
-      adj_step_f64_kernel<MODEL><<<adj_grid(g), dim3(kABX, kABY), 0, st>>>((const double*)fbuf,
-                                                                          (const double*)lam_next, (double*)lam, g, c);
+      const dim3 grid((g.nx + kAFX - 1) / kAFX, (g.ny + kAFY - 1) / kAFY);
+      return launch_step_kernel(adj_step_f64_kernel<MODEL>, grid, dim3(kAFX, kAFY), 0, st, (const double*)fbuf,
+                                (const double*)lam_next, (double*)lam, g, c);
     } else {
       adj_step_kernel<MODEL, PREC><<<adj_grid(g), dim3(kABX, kABY), 0, st>>>((const S*)fbuf, (const T*)lam_next,
                                                                             (T*)lam, g, c);
