@@ -75,7 +75,7 @@ struct Op {
 OLBM_EMU_HD Op digits(i64 v) {
   Op o;
   o.l = (int32_t)v;
-  o.h = (int32_t)((v + 0x80000000ll) >> 32);
+  o.h = (int32_t)(v >> 32) + (int32_t)((uint32_t)v >> 31);  // one shift-and-add instruction
   return o;
 }
 
@@ -133,7 +133,7 @@ OLBM_EMU_HD u64 uwide(uint32_t a, uint32_t b) {
 // dropped a.l b.l is at most a quarter unit of the result; the floor is one unit.
 template <int F, int G> OLBM_EMU_HD Fx<F + G - 64> operator*(FxOp<F> a, FxOp<G> b) {
   const i64 c = wide(a.o.l, b.o.h, wide(a.o.h, b.o.l));
-  return Fx<F + G - 64>{wide(a.o.h, b.o.h) + (c >> 32)};
+  return Fx<F + G - 64>{wide(a.o.h, b.o.h) + (i64)(int32_t)(c >> 32)};
 }
 template <int F> OLBM_EMU_HD Fx<2 * F - 64> square(FxOp<F> a) {
   return Fx<2 * F - 64>{wide(a.o.h, a.o.h) + (wide(a.o.h, a.o.l) >> 31)};

@@ -52,7 +52,8 @@ constexpr int kDfJoin = OLBM_DF_JOIN;
 // producer waits, their consumers touch global memory only after its copies); the
 // kernels that load through L1 signal after their own wait, so that no grid
 // before the previous one is still reading when the next one starts, and use plain
-// loads (the read-only path is not for data written while a grid is resident).
+// loads (the read-only path is not for data written while a grid is resident, so
+// their source pointers carry no __restrict__).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ double ld_plain(const double* p) {
@@ -353,9 +354,51 @@ template <int MODEL, int PREC, bool DIAG, bool PAIRS, bool CG = false> struct Co
     }
   }
 
+  // FP64 storage: the rows of a column in fixed point; returns the rows it left out. Byte
+  // offsets inside a plane as OFF: 32 bits where a plane is below 4 GiB, so that the nine
+  // loads and stores of a node take a uniform base and one 32-bit offset each instead of a
+  // 64-bit address (CG: for data written earlier in the same launch).
+  template <typename OFF>
+  __device__ static __forceinline__ unsigned long long run_fixed(const double* src, double* dst, const Geometry& g,
+                                                                 const fx::Coefs& c, int x, int xm, int xp, int y0,
+                                                                 int dy, int rows, FixedDiagAcc& facc) {
+    const OFF col[3] = {(OFF)xp * 8, (OFF)x * 8, (OFF)xm * 8};  // by c_ix + 1: the column x - c_ix
+    const OFF pitch = (OFF)g.pitch * 8;
+    auto load = [&](int y, double (&f)[9]) {
+      const OFF row[3] = {(OFF)(y == g.ny - 1 ? 0 : y + 1) * pitch, (OFF)y * pitch,
+                          (OFF)(y == 0 ? g.ny - 1 : y - 1) * pitch};
+#pragma unroll
+      for (int i = 0; i < 9; ++i) {
+        const char* plane = reinterpret_cast<const char*>(src + i * g.plane);
+        const double* p = reinterpret_cast<const double*>(plane + (OFF)(row[cy_of(i) + 1] + col[cx_of(i) + 1]));
+        f[i] = CG ? __ldcg(p) : *p;
+      }
+    };
+    unsigned long long left = 0;
+    double f[9];
+    int y = y0;
+    if (y < g.ny) load(y, f);
+    for (int r = 0; r < rows && y < g.ny; ++r, y += dy) {
+      const OFF q = (OFF)y * pitch + (OFF)x * 8;
+      const bool done = collide_fixed<MODEL>(
+          f, c,
+          [&](const FixedMoments& m) {
+            if constexpr (DIAG) facc.add(m);
+          },
+          [&](double (&h)[9]) {
+            if ((r + 1 < rows) && (y + dy < g.ny)) load(y + dy, h);
+          },
+          [&](int i, double v) {
+            *reinterpret_cast<double*>(reinterpret_cast<char*>(dst + i * g.plane) + q) = v;
+          });
+      left |= done ? 0ull : 1ull << r;
+    }
+    return left;
+  }
+
   // FIXED (FP64 storage): the fixed-point collision, which needs c.fixed.on.
   template <bool FIXED>
-  __device__ static __forceinline__ void run(const S* __restrict__ src, S* __restrict__ dst, const Geometry& g,
+  __device__ static __forceinline__ void run(const S* src, S* dst, const Geometry& g,
                                              const Coef<CT>& c, int x, int y0, int dy, int rows,
                                              DiagAcc<CT>& acc, FixedDiagAcc& facc) {
     if (x >= g.nx) return;
@@ -371,24 +414,9 @@ template <int MODEL, int PREC, bool DIAG, bool PAIRS, bool CG = false> struct Co
       // converted; then the rows it left out (bit r of `left`; rows <= 64) in the form's
       // own arithmetic.
       static_assert(PREC == 0 || PREC == 3, "the fixed-point collision is for FP64 storage");
-      using Raw = Column<MODEL, 0, DIAG, false, CG>;
-      unsigned long long left = 0;
-      double f[9];
-      int y = y0;
-      if (y < g.ny) Raw::pull(src, g, x, xm, xp, y, f);
-      for (int r = 0; r < rows && y < g.ny; ++r, y += dy) {
-        double* q = dst + (long long)y * g.pitch + x;
-        const bool done = collide_fixed<MODEL>(
-            f, c.fixed,
-            [&](const FixedMoments& m) {
-              if constexpr (DIAG) facc.add(m);
-            },
-            [&](double (&h)[9]) {
-              if ((r + 1 < rows) && (y + dy < g.ny)) Raw::pull(src, g, x, xm, xp, y + dy, h);
-            },
-            [&](int i, double v) { q[i * g.plane] = v; });
-        left |= done ? 0ull : 1ull << r;
-      }
+      const unsigned long long left =
+          g.plane < (1LL << 29) ? run_fixed<unsigned>(src, dst, g, c.fixed, x, xm, xp, y0, dy, rows, facc)
+                                : run_fixed<unsigned long long>(src, dst, g, c.fixed, x, xm, xp, y0, dy, rows, facc);
       if (__any_sync(__activemask(), left != 0)) {
         DiagAcc<CT> rest;  // (acc itself stays in registers: its address goes nowhere)
         run_float(src, dst, g, c, x, xm, xp, y0, dy, rows, left, rest);
@@ -455,8 +483,8 @@ template <int MODEL, int PREC, bool DIAG, bool PAIRS, bool CG = false> struct Co
 // kinetic energy and the number of nodes whose pulled populations do not sum to
 // a finite value go to partials[block * 5 + k].
 template <int MODEL, int PREC, bool DIAG, bool PAIRS, bool FIXED = false>
-__device__ __forceinline__ void step_body(const typename Form<PREC>::S* __restrict__ src,
-                                          typename Form<PREC>::S* __restrict__ dst, const Geometry& g,
+__device__ __forceinline__ void step_body(const typename Form<PREC>::S* src, typename Form<PREC>::S* dst,
+                                          const Geometry& g,
                                           const Coef<typename Column<MODEL, PREC, DIAG, PAIRS>::CT>& c,
                                           double* __restrict__ partials, int rows) {
   using Col = Column<MODEL, PREC, DIAG, PAIRS>;
@@ -492,7 +520,7 @@ __global__ void __launch_bounds__(512) step_kernel(const typename Form<PREC>::S*
 #define OLBM_DF_MAXNREG 96
 #endif
 template <int MODEL, bool DIAG, bool FIXED>
-__global__ void __maxnreg__(OLBM_DF_MAXNREG) step_kernel_df(const double* __restrict__ src, double* __restrict__ dst,
+__global__ void __maxnreg__(OLBM_DF_MAXNREG) step_kernel_df(const double* src, double* dst,
                                                       Geometry g, Coef<df64> c,
                                                       double* __restrict__ partials, int rows) {
   step_body<MODEL, 3, DIAG, false, FIXED>(src, dst, g, c, partials, rows);
@@ -509,7 +537,7 @@ __global__ void __maxnreg__(OLBM_DF_MAXNREG) step_kernel_df(const double* __rest
 #define OLBM_F64_MAXNREG 96
 #endif
 template <int MODEL, bool DIAG>
-__global__ void __maxnreg__(OLBM_F64_MAXNREG) step_kernel_f64(const double* __restrict__ src, double* __restrict__ dst, Geometry g,
+__global__ void __maxnreg__(OLBM_F64_MAXNREG) step_kernel_f64(const double* src, double* dst, Geometry g,
                                                 Coef<double> c, double* __restrict__ partials, int rows) {
   step_body<MODEL, 0, DIAG, false, true>(src, dst, g, c, partials, rows);
 }
