@@ -154,9 +154,9 @@ cudaError_t launch_diag(const lbm_ctx* c, cudaStream_t st) {
   const void* src = c->buf[c->cur];
   switch (c->prec) {
     case LBM_F64:
-    case LBM_F64_DF: return olbm::launch_diag_f64(src, c->g, c->rho_ref, c->d_parts[0], st);
-    case LBM_F32_SHIFT: return olbm::launch_diag_f32(src, c->g, c->rho_ref, c->d_parts[0], st);
-    default: return olbm::launch_diag_f16(src, c->g, c->rho_ref, c->d_parts[0], st);
+    case LBM_F64_DF: return olbm::launch_diag_f64(src, c->g, c->rho_ref, c->d_parts, st);
+    case LBM_F32_SHIFT: return olbm::launch_diag_f32(src, c->g, c->rho_ref, c->d_parts, st);
+    default: return olbm::launch_diag_f16(src, c->g, c->rho_ref, c->d_parts, st);
   }
 }
 
@@ -174,8 +174,8 @@ void free_ctx(lbm_ctx* c) {
     cudaFree(c->buf[0]);
     cudaFree(c->buf[1]);
   }
-  for (int b = 0; b < lbm_ctx::kParts; ++b) {
-    cudaFree(c->d_parts[b]);
+  cudaFree(c->d_parts);
+  for (int b = 0; b < lbm_ctx::kGroups; ++b) {
     if (c->ev_step[b]) cudaEventDestroy(c->ev_step[b]);
     if (c->ev_fin[b]) cudaEventDestroy(c->ev_fin[b]);
   }
@@ -254,7 +254,8 @@ int lbm_create_ex(int nx, int ny, double theta, double tau, int model, int prec,
     for (int w = 0; w < 2; ++w) c->tile[w] = olbm::tile_plan(c->g, prec, theta, tau, sms, w != 0);
   // (a cut into tiles has at most two an SM)
   // (diagnosed steps take at least as many rows, so no more partials, unless one row is all there is)
-  c->parts_cap = std::max({c->nparts, olbm::node_blocks(c->g), 2LL * sms});
+  c->parts_cap = std::max(c->nparts, 2LL * sms);
+  c->parts_total = std::max(c->parts_cap * lbm_ctx::kGroups * olbm::kFinalJobs, olbm::node_blocks(c->g));
 
   if (d_pop_buffers) {
     c->own_buffers = false;
@@ -270,9 +271,7 @@ int lbm_create_ex(int nx, int ny, double theta, double tau, int model, int prec,
       }
     }
   }
-  for (int b = 0; b < lbm_ctx::kParts && e == cudaSuccess; ++b)
-    e = cudaMalloc(&c->d_parts[b], sizeof(double) * 5 * (size_t)c->parts_cap);
-  if (e != cudaSuccess ||
+  if ((e = cudaMalloc(&c->d_parts, sizeof(double) * 5 * (size_t)c->parts_total)) != cudaSuccess ||
       (e = cudaMalloc(&c->d_diag, sizeof(double) * 6)) != cudaSuccess ||
       (e = cudaMalloc(&c->d_diag_now, sizeof(double) * 6)) != cudaSuccess ||
       (e = cudaMalloc(&c->d_sticky, sizeof(unsigned long long))) != cudaSuccess ||
@@ -283,7 +282,7 @@ int lbm_create_ex(int nx, int ny, double theta, double tau, int model, int prec,
     return fail(nullptr, LBM_ENOMEM, "cudaMalloc: %s", cudaGetErrorString(e));
   }
   e = cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking);
-  for (int b = 0; b < lbm_ctx::kParts && e == cudaSuccess; ++b) {
+  for (int b = 0; b < lbm_ctx::kGroups && e == cudaSuccess; ++b) {
     e = cudaEventCreateWithFlags(&c->ev_step[b], cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_fin[b], cudaEventDisableTiming);
   }
@@ -478,34 +477,48 @@ int lbm_step(lbm_ctx* ctx, int n) {
   a.theta = ctx->theta;
   a.tau = ctx->tau;
   a.rho_ref = ctx->rho_ref;
-  a.partials = ctx->d_parts[0];
+  a.partials = ctx->d_parts;
   a.cfg = ctx->cfg;
   a.err = ctx->d_err;
   a.sched = ctx->d_sched;
   long long used = ctx->nparts;
   a.parts_used = &used;
-  int joined = -1;  // partials buffer whose final sum was launched last (-1: none in this call)
-  // The next free partials buffer (waiting for its previous final sum), or null.
-  auto take = [&](bool diag, int& b) -> cudaError_t {
-    b = -1;
-    if (!diag) return cudaSuccess;
-    b = ctx->pbuf;
-    ctx->pbuf = (ctx->pbuf + 1) % lbm_ctx::kParts;
-    return ctx->fin_pending[b] ? cudaStreamWaitEvent(ctx->stream, ctx->ev_fin[b], 0) : cudaSuccess;
-  };
-  // The final sum of buffer b's partials (step time t) on the side stream, beside the next step.
-  auto finish = [&](int b, long long t) -> cudaError_t {
-    cudaError_t e;
-    if ((e = cudaEventRecord(ctx->ev_step[b], ctx->stream)) != cudaSuccess ||
-        (e = cudaStreamWaitEvent(ctx->side, ctx->ev_step[b], 0)) != cudaSuccess ||
-        (e = olbm::launch_finalize(ctx->d_parts[b], (int)used, ctx->rho_ref, nodes_of(ctx), t, ctx->d_diag,
-                                   ctx->d_sticky, ctx->side)) != cudaSuccess ||
-        (e = cudaEventRecord(ctx->ev_fin[b], ctx->side)) != cudaSuccess)
+  // Diagnosed steps whose partials wait for their final sum, in the buffers of group `group`.
+  olbm::FinalJobs jobs;
+  int group = 0, joined = -1;  // joined: the group summed last on the side stream (-1: none in this call)
+  bool pending[lbm_ctx::kGroups] = {};
+  // Their final sums: on the side stream, beside the next steps, or, at the end of a call that
+  // has none there, on `stream` (no events).
+  auto sum_group = [&](bool end) -> cudaError_t {
+    if (jobs.count == 0) return cudaSuccess;
+    const bool aside = !end || joined >= 0;
+    cudaError_t e = cudaSuccess;
+    if (aside && ((e = cudaEventRecord(ctx->ev_step[group], ctx->stream)) != cudaSuccess ||
+                  (e = cudaStreamWaitEvent(ctx->side, ctx->ev_step[group], 0)) != cudaSuccess))
       return e;
-    ctx->fin_pending[b] = true;
-    joined = b;
-    ctx->last_diag_t = t;
+    e = olbm::launch_finalize(jobs, ctx->rho_ref, nodes_of(ctx), ctx->d_diag, ctx->d_sticky,
+                              aside ? ctx->side : ctx->stream);
+    if (e != cudaSuccess) return e;
+    if (aside) {
+      if ((e = cudaEventRecord(ctx->ev_fin[group], ctx->side)) != cudaSuccess) return e;
+      pending[group] = true;
+      joined = group;
+    }
+    ctx->last_diag_t = jobs.t[jobs.count - 1];
+    jobs.count = 0;
+    group ^= 1;
     return cudaSuccess;
+  };
+  // Room for `need` more diagnosed steps in the current group.
+  auto reserve = [&](int need) -> cudaError_t {
+    cudaError_t e = cudaSuccess;
+    if (need == 0) return e;
+    if (jobs.count + need > olbm::kFinalJobs && (e = sum_group(false)) != cudaSuccess) return e;
+    if (jobs.count == 0 && pending[group]) {
+      pending[group] = false;
+      e = cudaStreamWaitEvent(ctx->stream, ctx->ev_fin[group], 0);
+    }
+    return e;
   };
   auto due = [&](long long t) { return ctx->diag_every > 0 && (t % ctx->diag_every) == 0; };
   a.wall_mask = ctx->d_wall_mask;
@@ -527,12 +540,10 @@ int lbm_step(lbm_ctx* ctx, int n) {
     used = ctx->nparts;
     a.cfg.rows = a.diag && ctx->diag_rows > 0 ? ctx->diag_rows : ctx->cfg.rows;
     if (a.cfg.rows != ctx->cfg.rows) used = olbm::step_blocks(ctx->g, a.cfg, ctx->prec);
-    int b1 = -1, b2 = -1;
-    cudaError_t e = take(a.diag, b1);
-    if (e == cudaSuccess) e = take(a.diag2, b2);
-    if (e != cudaSuccess) return cuda_fail(ctx, e, "lbm_step event wait");
-    a.partials = ctx->d_parts[b1 < 0 ? 0 : b1];
-    a.partials2 = ctx->d_parts[b2 < 0 ? 0 : b2];
+    cudaError_t e = reserve((a.diag ? 1 : 0) + (a.diag2 ? 1 : 0));
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "lbm_step diagnostics launch");
+    a.partials = ctx->parts(group, jobs.count);
+    a.partials2 = ctx->parts(group, jobs.count + (a.diag ? 1 : 0));
     e = many > 1 ? launch_tile(a, tile, many, ctx->prec, ctx->stream)
         : two    ? launch_step2(a, ctx->prec, ctx->stream)
                  : launch_step(a, ctx->prec, ctx->stream);
@@ -542,16 +553,17 @@ int lbm_step(lbm_ctx* ctx, int n) {
                              ctx->stream);
       if (e != cudaSuccess) return cuda_fail(ctx, e, "lbm_step walls launch");
     }
-    if (b1 >= 0 && (e = finish(b1, ctx->t)) != cudaSuccess) return cuda_fail(ctx, e, "lbm_step diagnostics launch");
-    if (b2 >= 0 && (e = finish(b2, ctx->t + 1)) != cudaSuccess)
-      return cuda_fail(ctx, e, "lbm_step diagnostics launch");
+    if (a.diag) jobs.add(a.partials, used, ctx->t);
+    if (a.diag2) jobs.add(a.partials2, used, ctx->t + 1);
     ctx->cur ^= 1;
     const int done = many > 1 ? many : (two ? 2 : 1);
     ctx->t += done;
     k += done;
   }
+  cudaError_t e = sum_group(true);
+  if (e != cudaSuccess) return cuda_fail(ctx, e, "lbm_step diagnostics launch");
   if (joined >= 0) {  // everything queued on `stream` after this call follows the final sums
-    cudaError_t e = cudaStreamWaitEvent(ctx->stream, ctx->ev_fin[joined], 0);
+    e = cudaStreamWaitEvent(ctx->stream, ctx->ev_fin[joined], 0);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "lbm_step join");
   }
   return LBM_OK;
@@ -598,9 +610,9 @@ int lbm_diagnostics(lbm_ctx* ctx, double* h_out5) {
   if (!h_out5) return fail(ctx, LBM_EINVAL, "lbm_diagnostics: NULL output");
   if (!ctx->initialised) return fail(ctx, LBM_ESTATE, "lbm_diagnostics before lbm_init / lbm_set_state");
   cudaError_t e = launch_diag(ctx, ctx->stream);
-  if (e == cudaSuccess)
-    e = olbm::launch_finalize(ctx->d_parts[0], (int)olbm::diag_blocks(ctx->g), ctx->rho_ref, nodes_of(ctx), ctx->t,
-                              ctx->d_diag_now, nullptr, ctx->stream);
+  olbm::FinalJobs job;
+  job.add(ctx->d_parts, olbm::diag_blocks(ctx->g), ctx->t);
+  if (e == cudaSuccess) e = olbm::launch_finalize(job, ctx->rho_ref, nodes_of(ctx), ctx->d_diag_now, nullptr, ctx->stream);
   double d[6];
   if (e == cudaSuccess) e = cudaMemcpyAsync(d, ctx->d_diag_now, sizeof(d), cudaMemcpyDeviceToHost, ctx->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
@@ -727,18 +739,15 @@ int lbm_set_launch_ex(lbm_ctx* ctx, int kind, int bx, int by, int rows) {
     cudaError_t e = cudaStreamSynchronize(ctx->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->side);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "lbm_set_launch sync");
-    double* p[lbm_ctx::kParts] = {};
-    for (int b = 0; b < lbm_ctx::kParts && e == cudaSuccess; ++b)
-      e = cudaMalloc(&p[b], sizeof(double) * 5 * (size_t)need);
-    if (e != cudaSuccess) {
-      for (int b = 0; b < lbm_ctx::kParts; ++b) cudaFree(p[b]);
+    double* p = nullptr;
+    const long long total = std::max(need * lbm_ctx::kGroups * olbm::kFinalJobs, ctx->parts_total);
+    if ((e = cudaMalloc(&p, sizeof(double) * 5 * (size_t)total)) != cudaSuccess) {
       cudaGetLastError();
       return fail(ctx, LBM_ENOMEM, "lbm_set_launch: %s", cudaGetErrorString(e));
     }
-    for (int b = 0; b < lbm_ctx::kParts; ++b) {
-      cudaFree(ctx->d_parts[b]);
-      ctx->d_parts[b] = p[b];
-    }
+    cudaFree(ctx->d_parts);
+    ctx->d_parts = p;
+    ctx->parts_total = total;
     ctx->parts_cap = need;
   }
   ctx->cfg = k;

@@ -22,22 +22,22 @@ struct lbm_ctx {
   int diag_rows = 0;  // rows of a diagnosed step under the default FP64 launch (0: as cfg)
   // several steps a launch on small lattices, without and with walls; off once lbm_set_launch chose a shape
   olbm::TilesPlan tile[2]{};
-  // Per-block diagnostics partials, kParts buffers of parts_cap blocks each (d_parts[0]
-  // also serves lbm_diagnostics). Consecutive diagnosed steps take the buffers in turn,
-  // and the final sum of step t runs on a second stream while later steps run; lbm_step
-  // joins that stream back into `stream` before it returns. A two-step launch takes two
-  // buffers at once, so the next launch's buffers are never the ones still being summed.
-  static constexpr int kParts = 4;
-  double* d_parts[kParts] = {nullptr, nullptr, nullptr, nullptr};
-  long long nparts = 0;      // partials the step kernel writes under cfg
-  long long parts_cap = 0;   // partials allocated (each buffer)
+  // Per-block diagnostics partials: kGroups groups of olbm::kFinalJobs buffers of parts_cap
+  // blocks each, in one allocation (its start also serves lbm_diagnostics). Diagnosed steps
+  // fill a group's buffers in turn; the final sums of a full group are one launch on a second
+  // stream, while later steps fill the other group, and lbm_step joins that stream back
+  // into `stream` before it returns (a call that fills no group sums on `stream` itself).
+  static constexpr int kGroups = 2;
+  double* d_parts = nullptr;
+  double* parts(int group, int k) const { return d_parts + 5 * parts_cap * (group * olbm::kFinalJobs + k); }
+  long long nparts = 0;       // partials the step kernel writes under cfg
+  long long parts_cap = 0;    // partials of one buffer
+  long long parts_total = 0;  // partials allocated
   cudaStream_t side = nullptr;
-  cudaEvent_t ev_step[kParts] = {};  // partials of buffer b written (on `stream`)
-  cudaEvent_t ev_fin[kParts] = {};   // partials of buffer b summed (on `side`)
+  cudaEvent_t ev_step[kGroups] = {};  // partials of the group written (on `stream`)
+  cudaEvent_t ev_fin[kGroups] = {};   // partials of the group summed (on `side`)
   cudaEvent_t ev_io = nullptr;                  // lbm_run_host: moments written (on `stream`)
   cudaEvent_t ev_rebind = nullptr;              // lbm_set_stream: end of the old stream's work
-  bool fin_pending[kParts] = {};
-  int pbuf = 0;  // partials buffer of the next diagnosed step (0 .. kParts - 1)
   double* d_diag = nullptr;      // [6] latest fused diagnostics (out5 + time)
   double* d_diag_now = nullptr;  // [6] scratch of lbm_diagnostics
   unsigned long long* d_sticky = nullptr;

@@ -92,7 +92,21 @@ cudaError_t launch_step2_f16(const StepArgs& a, cudaStream_t st);
 // Record a message for lbm_last_error(NULL) on this thread; returns status.
 int set_thread_error(int status, const char* fmt, ...);
 
-cudaError_t launch_finalize(const double* partials, int nparts, double rho_ref, long long nodes, long long t,
-                            double* out, unsigned long long* sticky, cudaStream_t st);
+// Final sums of the block partials of up to kFinalJobs diagnosed steps in one launch, one
+// block a step; the last of them goes to out[0..5], the non-finite nodes of all are added to
+// *sticky (may be null).
+constexpr int kFinalJobs = 8;
+struct FinalJobs {
+  const double* partials[kFinalJobs];
+  int nparts[kFinalJobs];
+  long long t[kFinalJobs];
+  int count = 0;
+  void add(const double* p, long long n, long long time) {
+    partials[count] = p, nparts[count] = (int)n, t[count] = time;
+    ++count;
+  }
+};
+cudaError_t launch_finalize(const FinalJobs& jobs, double rho_ref, long long nodes, double* out,
+                            unsigned long long* sticky, cudaStream_t st);
 
 }  // namespace olbm

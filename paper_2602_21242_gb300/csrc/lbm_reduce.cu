@@ -41,14 +41,18 @@ long long step2_blocks(const Geometry& g, const LaunchCfg& k, int prec) {
 #endif
 int stream_ctas_per_sm(int) { return OLBM_STREAM_CTAS; }
 
-// Fixed-order final sum of the block partials: out[0..4] as in lbm_diagnostics
-// (mass gets rho_ref for every finite node), out[5] = t; non-finite nodes are
-// added to *sticky.
+// Fixed-order final sums of the block partials, one block a diagnosed step: out[0..4] as in
+// lbm_diagnostics (mass gets rho_ref for every finite node), out[5] = t of the last step;
+// non-finite nodes of every step are added to *sticky.
+//
+// A sum alone is a launch, two events and a stream wait for the host and breaks the chain of
+// programmatically launched steps; on small lattices that was most of a diagnosed step (@@).
 constexpr int kFinalThreads = 512;
-__global__ void __launch_bounds__(kFinalThreads) finalize_kernel(const double* __restrict__ partials, int nparts,
-                                                                 double rho_ref, long long nodes, long long t,
+__global__ void __launch_bounds__(kFinalThreads) finalize_kernel(FinalJobs jobs, double rho_ref, long long nodes,
                                                                  double* __restrict__ out,
                                                                  unsigned long long* __restrict__ sticky) {
+  const double* __restrict__ partials = jobs.partials[blockIdx.x];
+  const int nparts = jobs.nparts[blockIdx.x];
   double v[kNDiag] = {0.0, 0.0, 0.0, 0.0, 0.0};
   for (int j = threadIdx.x; j < nparts; j += kFinalThreads)
 #pragma unroll
@@ -57,19 +61,21 @@ __global__ void __launch_bounds__(kFinalThreads) finalize_kernel(const double* _
   block_sum<kNDiag, kFinalThreads>(v, tot);
   if (threadIdx.x == 0) {
     const double bad = tot[4];
-    out[0] = tot[0] + rho_ref * (double)(nodes - (long long)bad);
-    out[1] = tot[1];
-    out[2] = tot[2];
-    out[3] = tot[3];
-    out[4] = bad;
-    out[5] = (double)t;
-    if (bad > 0.0 && sticky != nullptr) *sticky += (unsigned long long)bad;
+    if (blockIdx.x + 1 == gridDim.x) {
+      out[0] = tot[0] + rho_ref * (double)(nodes - (long long)bad);
+      out[1] = tot[1];
+      out[2] = tot[2];
+      out[3] = tot[3];
+      out[4] = bad;
+      out[5] = (double)jobs.t[blockIdx.x];
+    }
+    if (bad > 0.0 && sticky != nullptr) atomicAdd(sticky, (unsigned long long)bad);
   }
 }
 
-cudaError_t launch_finalize(const double* partials, int nparts, double rho_ref, long long nodes, long long t,
-                            double* out, unsigned long long* sticky, cudaStream_t st) {
-  finalize_kernel<<<1, kFinalThreads, 0, st>>>(partials, nparts, rho_ref, nodes, t, out, sticky);
+cudaError_t launch_finalize(const FinalJobs& jobs, double rho_ref, long long nodes, double* out,
+                            unsigned long long* sticky, cudaStream_t st) {
+  finalize_kernel<<<jobs.count, kFinalThreads, 0, st>>>(jobs, rho_ref, nodes, out, sticky);
   return cudaGetLastError();
 }
 
