@@ -116,12 +116,18 @@ olbm::LaunchCfg default_cfg(int prec, const olbm::Geometry& g, int sms) {
   return k;
 }
 
-// Rows per thread of a diagnosed FP64 step under the default launch: at least 6 CTAs per SM
-// where the plain step has 20, because one block sums the CTAs' partials beside the next
-// step (512^2, diagnostics every step: 37.0 us a step with 1 row and 4096 partials).
+// Rows per thread of a diagnosed FP64 step under the default launch. A CTA's reduction costs about as
+// much as a row of its threads, so fewer and taller CTAs than the plain step's: at least 17
+// per SM (their last wave is short beside them), but no fewer than five rows while that
+// leaves 4.4 per SM (one wave of the five resident, not quite full). us a step, diagnostics every step, by rows: 2048^2 12 rows 133.4,
+// 32 139.6, 4 139.3; 1024^2 6 rows 39.8, 3 41.3, 12 42.8; 512^2 3 rows 13.1, 1 15.2, 6 15.2; 400^2
+// 2 rows 9.9, 1 11.3, 3 12.6.
 int diag_rows(const olbm::Geometry& g, olbm::LaunchCfg k, int prec, int sms) {
-  for (k.rows = 32; k.rows > 1 && olbm::step_blocks(g, k, prec) < 6LL * sms;) --k.rows;
-  return k.rows;
+  auto rows_for = [&](double ctas) {
+    for (k.rows = 32; k.rows > 1 && olbm::step_blocks(g, k, prec) < ctas * sms;) --k.rows;
+    return k.rows;
+  };
+  return std::max(rows_for(17.0), std::min(5, rows_for(4.4)));
 }
 
 cudaError_t launch_step(const olbm::StepArgs& a, int prec, cudaStream_t st) {

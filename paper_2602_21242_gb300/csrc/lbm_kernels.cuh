@@ -196,11 +196,6 @@ struct Sum96 {
         : "+r"(lo), "+r"(mid), "+r"(hi)
         : "r"((unsigned)v), "r"((unsigned)(v >> 32)), "r"((int)(v >> 63)));
   }
-  // The sum in units of 2^-60, the low 64 bits taken as a signed number.
-  __device__ __forceinline__ double value() const {
-    const long long low = (long long)(((unsigned long long)mid << 32) | lo);
-    return fma((double)(hi + (int)(mid >> 31)), 16.0, (double)low * 0x1p-60);
-  }
 };
 struct FixedDiagAcc {
   Sum96 s[4];
@@ -211,6 +206,71 @@ struct FixedDiagAcc {
     s[3].add(m.ke2);
   }
 };
+// The same over a block, with the accumulators v and bad of the nodes outside the fixed-point
+// path (kinetic energies already halved): out5 receives the totals (threads 0 to 4 write).
+//
+// An FP64 reduction (conversions, products and five butterfly steps of four sums) holds the FP64 pipe
+// for about 2500 cycles a block of 128, which was most of a diagnosed step where a thread has few
+// rows. So the integer sums stay integers: digits of 26 bits, each summed over the warp by
+// one instruction (32 digits fit 32 bits; sums up to 2^78 units, 2^18 a thread, fit three digits),
+// then over the warps in 64 bits, and are rounded once at the end. Warps without a node in
+// floating point skip its butterfly. 2042 x 106 FP64, diagnostics every step:
+// 31.1 -> 13.9 us a step (12.5 with the rows of diag_rows); 256^2 14.0 -> 7.0.
+struct FixedDiagShared {
+  int digit[kMaxWarps][12];
+  double v[kMaxWarps][4];
+  int bad[kMaxWarps];  // -1: no node of the warp in floating point
+};
+__device__ __forceinline__ void block_diag_fixed(double (&v)[4], int bad, const FixedDiagAcc& f, double* out5) {
+  __shared__ FixedDiagShared sh;
+  unsigned long long any = (unsigned long long)bad;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) any |= (unsigned long long)__double_as_longlong(v[k]);
+  const int tid = threadIdx.x + blockDim.x * threadIdx.y, warp = tid >> 5;
+  const bool floats = __any_sync(0xffffffffu, any != 0);
+  if (floats) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+      bad += __shfl_xor_sync(0xffffffffu, bad, o);
+    }
+  }
+  int d[12];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const unsigned mask = (1u << 26) - 1u;
+    d[3 * k] = (int)__reduce_add_sync(0xffffffffu, f.s[k].lo & mask);
+    d[3 * k + 1] = (int)__reduce_add_sync(0xffffffffu, __funnelshift_r(f.s[k].lo, f.s[k].mid, 26) & mask);
+    d[3 * k + 2] = __reduce_add_sync(0xffffffffu, (int)__funnelshift_l(f.s[k].mid, (unsigned)f.s[k].hi, 12));
+  }
+  if ((tid & 31) == 0) {
+#pragma unroll
+    for (int k = 0; k < 12; ++k) sh.digit[warp][k] = d[k];
+    if (floats) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) sh.v[warp][k] = v[k];
+    }
+    sh.bad[warp] = floats ? bad : -1;
+  }
+  __syncthreads();
+  const int nw = (blockDim.x * blockDim.y) >> 5;
+  if (tid < 4) {
+    long long a = 0, b = 0, c = 0;
+    double t = 0.0;
+    for (int w = 0; w < nw; ++w) {
+      a += (unsigned)sh.digit[w][3 * tid], b += (unsigned)sh.digit[w][3 * tid + 1], c += sh.digit[w][3 * tid + 2];
+      if (sh.bad[w] >= 0) t += sh.v[w][tid];
+    }
+    a += b << 26, c += a >> 52;  // (a < 2^62)
+    const double sum = fma((double)c, 0x1p-8, (double)(a & ((1LL << 52) - 1)) * 0x1p-60);  // rounded once
+    out5[tid] = t + (tid == 3 ? 0.5 * sum : sum);
+  } else if (tid == 4) {
+    int n = 0;
+    for (int w = 0; w < nw; ++w) n += max(sh.bad[w], 0);
+    out5[4] = (double)n;
+  }
+}
 // Packed pairs accumulate into four FP32 scalars: both nodes of a pair go into
 // the same sums, which holds four registers fewer through the collision than
 // packed sums would (measured on the FP16 form at 4096^2 with diagnostics every
@@ -252,9 +312,11 @@ __device__ __forceinline__ void block_diag_acc(DiagAcc<CT>& a, double* out5, con
     for (int k = 0; k < 4; ++k) {
       if constexpr (std::is_same<CT, df64>::value) v[k] = join_f64(a.v[k]);
       else v[k] = a.v[k];
-      if (fixed != nullptr) v[k] += fixed->s[k].value() * (k == 3 ? 0.5 : 1.0);
     }
-    block_diag<double>(v, a.bad, out5);
+    if (fixed != nullptr)
+      block_diag_fixed(v, a.bad, *fixed, out5);
+    else
+      block_diag<double>(v, a.bad, out5);
   } else {
     block_diag<CT>(a.v, a.bad, out5);
   }
@@ -616,9 +678,7 @@ __device__ __forceinline__ void diag_node(const typename Form<PREC>::S* __restri
 
 // Block totals of the accumulators of a diagnostics pass (sums and the count of nodes whose
 // populations do not sum to a finite value) into p[0 .. 4].
-__device__ __forceinline__ void diag_store(double (&acc)[kNDiag], const FixedDiagAcc& facc, double* __restrict__ p) {
-#pragma unroll
-  for (int k = 0; k < 4; ++k) acc[k] += facc.s[k].value() * (k == 3 ? 0.5 : 1.0);
+__device__ __forceinline__ void diag_store(double (&acc)[kNDiag], double* __restrict__ p) {
   double tot[kNDiag];
   block_sum<kNDiag, kNT>(acc, tot);
   if (threadIdx.x == 0 && threadIdx.y == 0) {
@@ -666,7 +726,13 @@ __global__ void __launch_bounds__(kNT) diag_kernel(const typename Form<PREC>::S*
       diag_node<PREC>(src, g, x, y, rho_ref, acc);
     }
   }
-  diag_store(acc, facc, partials + (long long)(blockIdx.y * gridDim.x + blockIdx.x) * kNDiag);
+  double* const out = partials + (long long)(blockIdx.y * gridDim.x + blockIdx.x) * kNDiag;
+  if constexpr (PREC == 0) {
+    double v[4] = {acc[0], acc[1], acc[2], acc[3]};
+    block_diag_fixed(v, (int)acc[4], facc, out);
+  } else {
+    diag_store(acc, out);
+  }
 }
 
 // ------------------------------------------------------------------ init, moments, state copies

@@ -46,7 +46,8 @@ int stream_ctas_per_sm(int) { return OLBM_STREAM_CTAS; }
 // non-finite nodes of every step are added to *sticky.
 //
 // A sum alone is a launch, two events and a stream wait for the host and breaks the chain of
-// programmatically launched steps; on small lattices that was most of a diagnosed step (@@).
+// programmatically launched steps; on small lattices that was most of a diagnosed step
+// (64^2, diagnostics every step: FP32 10.9 -> 3.8 us, FP64 10.9 -> 5.3).
 constexpr int kFinalThreads = 512;
 __global__ void __launch_bounds__(kFinalThreads) finalize_kernel(FinalJobs jobs, double rho_ref, long long nodes,
                                                                  double* __restrict__ out,
