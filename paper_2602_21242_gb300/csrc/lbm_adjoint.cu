@@ -22,7 +22,33 @@ namespace olbm {
 
 constexpr int kABX = 32, kABY = 8;
 
-// lambda(n) from the cotangents of the final moments (any may be NULL = 0).
+// FP32 <-> FP64 conversions in integers for the values that are normal in FP32 (and +-0 for
+// widen), the instruction for the others: the same results, off the FP64 pipe.
+__device__ __forceinline__ double widen(float x) {
+  const unsigned b = __float_as_uint(x), m = b << 1;
+  if (m - (1u << 24) < (254u << 24))
+    return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7FFFFFFFu) >> 3) + (896u << 20))), (int)(b << 29));
+  return m == 0 ? __hiloint2double((int)b, 0) : (double)x;
+}
+__device__ __forceinline__ double widen(double x) { return x; }
+__device__ __forceinline__ double widen(df64 x) { return to_double(x); }
+template <typename T> __device__ __forceinline__ T narrow(double x);
+template <> __device__ __forceinline__ double narrow<double>(double x) { return x; }
+template <> __device__ __forceinline__ df64 narrow<df64>(double x) { return (df64)x; }
+template <> __device__ __forceinline__ float narrow<float>(double x) {  // to nearest, ties to even
+  const unsigned long long u = (unsigned long long)__double_as_longlong(x);
+  const unsigned hi = (unsigned)(u >> 32);
+  if (((hi & 0x7FFFFFFFu) >> 20) - 897u < 253u) {
+    const unsigned long long r = (u & 0x7FFFFFFFFFFFFFFFull) + 0x0FFFFFFFull + ((u >> 29) & 1u);
+    return __uint_as_float(((unsigned)(r >> 29) - (896u << 23)) | (hi & 0x80000000u));
+  }
+  return (float)x;
+}
+
+// lambda(n) from the cotangents of the final moments (any may be NULL = 0). Bound by the FP64 pipe
+// before (two divisions a cotangent, four operations a population, conversions: 185 us at 1024^2
+// in FP32); now the moments are summed in integers (pulled_sums), 1/rho is formed once and
+// the nine values are sums of three (65 us).
 template <int PREC>
 __global__ void __launch_bounds__(kABX* kABY) adj_seed_kernel(const typename Form<PREC>::S* __restrict__ fbuf,
                                                               Geometry g, double rho_ref,
@@ -33,23 +59,19 @@ __global__ void __launch_bounds__(kABX* kABY) adj_seed_kernel(const typename For
   using T = typename Form<PREC>::T;
   const int x = blockIdx.x * kABX + threadIdx.x, y = blockIdx.y * kABY + threadIdx.y;
   if (x >= g.nx || y >= g.ny) return;
-  long long o[9];
-  pull_offsets(x, y, g, o);
-  double m0 = 0.0, jx = 0.0, jy = 0.0;
-#pragma unroll
-  for (int i = 0; i < 9; ++i) {
-    const double v = to_double(fbuf[i * g.plane + o[i]]);
-    m0 += v;
-    jx += (double)cx_of(i) * v;
-    jy += (double)cy_of(i) * v;
-  }
-  const double rho = rho_ref + m0, ux = jx / rho, uy = jy / rho;
+  double m0, jx, jy;
+  pulled_sums<PREC == 3 ? 0 : PREC>(fbuf, g, x, y, m0, jx, jy);
+  const double rho = PREC == 1 ? rho_ref + m0 : m0;
+  // (the reciprocal of the collision takes densities in [2^-126, 2^126))
+  const double r = ((unsigned)__double2hiint(rho) >> 20) - 900u < 246u ? recip(rho) : 1.0 / rho;
+  const double ux = jx * r, uy = jy * r;
   const long long n = (long long)y * g.nx + x;
-  const double gr = g_rho ? g_rho[n] : 0.0, gx = g_ux ? g_ux[n] / rho : 0.0, gy = g_uy ? g_uy[n] / rho : 0.0;
-  const long long here = (long long)y * g.pitch + x;
+  const double gr = g_rho ? g_rho[n] : 0.0, gx = g_ux ? g_ux[n] * r : 0.0, gy = g_uy ? g_uy[n] * r : 0.0;
+  const double b = gr - (ux * gx + uy * gy), bp = b + gx, bm = b - gx;
+  T* const out = lam + (long long)y * g.pitch + x;
+  const double v[9] = {b, bp, b + gy, bm, b - gy, bp + gy, bm + gy, bm - gy, bp - gy};
 #pragma unroll
-  for (int i = 0; i < 9; ++i)
-    lam[i * g.plane + here] = (T)(gr + ((double)cx_of(i) - ux) * gx + ((double)cy_of(i) - uy) * gy);
+  for (int i = 0; i < 9; ++i) out[i * g.plane] = narrow<T>(v[i]);
 }
 
 // lambda(t)(x) = J_C(f(x, t))^T mu(x), mu_i(x) = lambda_i(t + 1)(x + c_i).
@@ -179,28 +201,37 @@ __global__ void __launch_bounds__(kAFX* kAFY, OLBM_ADJ_F64_MINB) adj_step_f64_ke
 // (nx even): f pulled as the forward pair kernels pull it, mu push-read as pairs
 // (the c_ix = 0 planes aligned, the others element by element), lambda stored
 // as aligned pairs.
-// Three blocks a SM (80 registers): the 1024^2 FP32 gradient's backward pass
-// 18.99 -> 18.04 ms (four blocks spill: 23.35 ms).
+// Three blocks a SM (80 registers): the 1024^2 FP32 gradient's backward pass of 500 steps
+// 18.99 -> 18.04 ms (four blocks spill: 23.35 ms). 20 us at 1024^2, 113 MB: near the bandwidth.
 #ifndef OLBM_ADJ_PAIR_MINB
 #define OLBM_ADJ_PAIR_MINB 3
 #endif
+// Launched with programmatic serialization, so its loads are plain ones after the wait (no
+// read-only loads, which may move above it).
+__device__ __forceinline__ f32x2 two_plain(const float* p0, const float* p1) { return f32x2(make_float2(*p0, *p1)); }
+__device__ __forceinline__ f32x2 pair_plain(const float* p) { return f32x2(*reinterpret_cast<const float2*>(p)); }
 template <int MODEL>
-__global__ void __launch_bounds__(kABX* kABY, OLBM_ADJ_PAIR_MINB) adj_step_pair_kernel(const float* __restrict__ fbuf,
-                                                                   const float* __restrict__ lam_next,
-                                                                   float* __restrict__ lam, Geometry g,
-                                                                   Coef<f32x2> c) {
+__global__ void __launch_bounds__(kABX* kABY, OLBM_ADJ_PAIR_MINB) adj_step_pair_kernel(const float* fbuf,
+                                                                                       const float* lam_next, float* lam,
+                                                                                       Geometry g, Coef<f32x2> c) {
   const int x = 2 * (blockIdx.x * kABX + threadIdx.x), y = blockIdx.y * kABY + threadIdx.y;
+  pdl_wait();
+  pdl_launch_dependents();
   if (x >= g.nx || y >= g.ny) return;
   const int xm = x == 0 ? g.nx - 1 : x - 1;           // x - 1, periodic
   const int xp = x + 2 >= g.nx ? x + 2 - g.nx : x + 2;  // x + 2, periodic
   f32x2 f[9], mu[9], out[9];
-  Column<MODEL, 1, false, true>::pull(fbuf, g, x, xm, xp, y, f);
+  const long long rows[3] = {(long long)(y == 0 ? g.ny - 1 : y - 1) * g.pitch, (long long)y * g.pitch,
+                             (long long)(y == g.ny - 1 ? 0 : y + 1) * g.pitch};  // y - 1, y, y + 1, periodic
 #pragma unroll
-  for (int i = 0; i < 9; ++i) {
-    int yd = y + cy_of(i);  // y + c_iy, periodic
-    yd = yd < 0 ? yd + g.ny : (yd >= g.ny ? yd - g.ny : yd);
-    const float* q = lam_next + i * g.plane + (long long)yd * g.pitch;
-    mu[i] = cx_of(i) == 0 ? ld_pair(q + x) : (cx_of(i) > 0 ? ld_two(q + x + 1, q + xp) : ld_two(q + xm, q + x));
+  for (int i = 0; i < 9; ++i) {  // f_i at x - c_i
+    const float* q = fbuf + i * g.plane + rows[1 - cy_of(i)];
+    f[i] = cx_of(i) == 0 ? pair_plain(q + x) : (cx_of(i) > 0 ? two_plain(q + xm, q + x) : two_plain(q + x + 1, q + xp));
+  }
+#pragma unroll
+  for (int i = 0; i < 9; ++i) {  // lambda_i at x + c_i
+    const float* q = lam_next + i * g.plane + rows[1 + cy_of(i)];
+    mu[i] = cx_of(i) == 0 ? pair_plain(q + x) : (cx_of(i) > 0 ? two_plain(q + x + 1, q + xp) : two_plain(q + xm, q + x));
   }
   collide_vjp<MODEL, true, f32x2>(f, mu, c, out);
   float* o = lam + (long long)y * g.pitch + x;
@@ -208,7 +239,11 @@ __global__ void __launch_bounds__(kABX* kABY, OLBM_ADJ_PAIR_MINB) adj_step_pair_
   for (int i = 0; i < 9; ++i) st_pair(o + i * g.plane, out[i]);
 }
 
-// Cotangents of (rho0, u0) from lambda(0), through f(x, 0) = f^eq(rho0(x), u0(x)).
+// Cotangents of (rho0, u0) from lambda(0), through f(x, 0) = f^eq(rho0(x), u0(x)). With the transposed
+// moments of an axis, M0 = l(0), M1 = (l(1) - l(-1)) / 2, M2 = (l(1) + l(-1)) / 2 - l(0), the
+// factor sum_b l(b) P(b) is M0 + v M1 + (theta + v^2) M2 and its derivative M1 + 2 v M2, first over b
+// for each a, then over a: about 45 FP64 operations a node, which bind it (85 before: 1024^2
+// in FP32 146 us, now 95).
 template <int PREC>
 __global__ void __launch_bounds__(kABX* kABY) adj_final_kernel(const typename Form<PREC>::T* __restrict__ lam,
                                                                Geometry g, double theta,
@@ -222,23 +257,25 @@ __global__ void __launch_bounds__(kABX* kABY) adj_final_kernel(const typename Fo
   if (x >= g.nx || y >= g.ny) return;
   const long long n = (long long)y * g.nx + x, here = (long long)y * g.pitch + x;
   const double rho = rho0[n], ux = ux0[n], uy = uy0[n];
-  const double px[3] = {0.5 * (theta + ux * ux - ux), 1.0 - theta - ux * ux, 0.5 * (theta + ux * ux + ux)};
-  const double py[3] = {0.5 * (theta + uy * uy - uy), 1.0 - theta - uy * uy, 0.5 * (theta + uy * uy + uy)};
-  const double dpx[3] = {ux - 0.5, -2.0 * ux, ux + 0.5};
-  const double dpy[3] = {uy - 0.5, -2.0 * uy, uy + 0.5};
-  double gr = 0.0, gx = 0.0, gy = 0.0;
+  double l[9];
 #pragma unroll
-  for (int a = -1; a <= 1; ++a)
+  for (int i = 0; i < 9; ++i) l[i] = widen(lam[i * g.plane + here]);
+  // per a: Y = sum_b l P_y(b), Z = sum_b l P_y'(b)
+  const double qx = fma(ux, ux, theta), qy = fma(uy, uy, theta), hx = 0.5 * ux, hy = 0.5 * uy, hqx = 0.5 * qx,
+               hqy = 0.5 * qy;
+  double Y[3], Z[3];
 #pragma unroll
-    for (int b = -1; b <= 1; ++b) {
-      const double l = to_double(lam[pop_index(a, b) * g.plane + here]);
-      gr += l * px[a + 1] * py[b + 1];
-      gx += l * dpx[a + 1] * py[b + 1];
-      gy += l * px[a + 1] * dpy[b + 1];
-    }
-  if (g_rho0) g_rho0[n] = gr;
-  if (g_ux0) g_ux0[n] = rho * gx;
-  if (g_uy0) g_uy0[n] = rho * gy;
+  for (int a = -1; a <= 1; ++a) {
+    const double l0 = l[pop_index(a, 0)], lp = l[pop_index(a, 1)], lm = l[pop_index(a, -1)];
+    const double d = lp - lm, s = (lp - l0) + (lm - l0);  // 2 M1, 2 M2
+    Y[a + 1] = fma(hqy, s, fma(hy, d, l0));
+    Z[a + 1] = fma(uy, s, 0.5 * d);
+  }
+  const double dY = Y[2] - Y[0], sY = (Y[2] - Y[1]) + (Y[0] - Y[1]);
+  const double dZ = Z[2] - Z[0], sZ = (Z[2] - Z[1]) + (Z[0] - Z[1]);
+  if (g_rho0) g_rho0[n] = fma(hqx, sY, fma(hx, dY, Y[1]));
+  if (g_ux0) g_ux0[n] = rho * fma(ux, sY, 0.5 * dY);
+  if (g_uy0) g_uy0[n] = rho * fma(hqx, sZ, fma(hx, dZ, Z[1]));
 }
 
 inline dim3 adj_grid(const Geometry& g) { return dim3((g.nx + kABX - 1) / kABX, (g.ny + kABY - 1) / kABY); }
@@ -259,9 +296,8 @@ template <int PREC> struct Adjoint {
     if constexpr (PREC == 1) {
       if (g.nx % 2 == 0) {
         const dim3 grid((g.nx / 2 + kABX - 1) / kABX, (g.ny + kABY - 1) / kABY);
-        adj_step_pair_kernel<MODEL><<<grid, dim3(kABX, kABY), 0, st>>>(
-            (const float*)fbuf, (const float*)lam_next, (float*)lam, g, make_coef<f32x2>(theta, tau, rho_ref));
-        return cudaGetLastError();
+        return launch_step_kernel(adj_step_pair_kernel<MODEL>, grid, dim3(kABX, kABY), 0, st, (const float*)fbuf,
+                                  (const float*)lam_next, (float*)lam, g, make_coef<f32x2>(theta, tau, rho_ref));
       }
     }
     if constexpr (PREC == 0) {
