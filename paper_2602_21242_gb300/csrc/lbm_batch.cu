@@ -104,6 +104,7 @@ struct lbm_batch {
   // the single steps of an odd count take the kind 1 tiles above
   int4* d_tiles2 = nullptr;
   int2* d_ranges2 = nullptr;
+  int rows = 0;  // tile rows of a small batch under the default shape (0: cfg.rows)
   int ntiles2 = 0;
   double* d_parts[kParts] = {};  // per-tile partials, max(ntiles, ntiles2) each
   double* d_diag = nullptr;  // n * 5, latest fused diagnostics
@@ -173,6 +174,9 @@ template <typename CT> void fill_desc(lbm_batch* b, std::vector<olbm::Desc<CT>>&
   }
 }
 
+// Tile rows of the launches (of lbm_batch_get_launch's shape at most).
+int rows_of(const lbm_batch* b) { return b->rows > 0 ? b->rows : b->cfg.rows; }
+
 // Tiles of cols x trows of every domain, domain after domain, and each domain's range.
 void cut_tiles(const lbm_batch* b, int cols, int trows, std::vector<int4>& tiles, std::vector<int2>& ranges) {
   tiles.clear();
@@ -186,21 +190,49 @@ void cut_tiles(const lbm_batch* b, int cols, int trows, std::vector<int4>& tiles
   }
 }
 
+// Default tiles: FP64 the column routine with 64 x 2 threads and up to 16 rows; FP16 the
+// bulk-copy pipeline on tiles of up to 32 rows; FP32 two steps a launch on tiles of up to 32 rows
+// (256 Taylor-Green domains N ~ U{64..512}, diagnostics every step: 113.3 GLUPS in graph
+// mode against 83.3 for the single-step pipeline; the persistent mode takes single steps
+// either way). A small batch takes shorter tiles, by the rows S of all its strips: a step of
+// few tiles lasts as long as one tile (23 us with 32 rows, 18 with 16 in FP64, however small the
+// batch). FP32 and FP16: S / 3 SMs, about one wave, while that is at most 18 rows, then at
+// least two waves; FP64: 17 CTAs an SM. us a step of 50, before -> now (best of 1 to 32
+// rows): 4 domains of 24 to 128, FP32 23.0 -> 3.5 (3.5), FP16 21.0 -> 3.1 (3.1), FP64 18.3 -> 4.7
+// (4.5); 20 of 40 to 200, 23.1 -> 8.1 (8.1), 22.0 -> 11.4 (10.6), 25.4 -> 18.6 (18.6); 64 of 96 to
+// 400, 57.8 -> 49.5 (47.8), 64.7 -> 62 (62), 164 (164).
+void default_tiles(lbm_batch* b) {
+  if (b->prec == LBM_F64) {
+    b->cfg.bx = 64, b->cfg.by = 2, b->cfg.rows = 16;
+  } else {
+    b->cfg.kind = b->prec == LBM_F32_SHIFT ? 2 : 1, b->cfg.bx = 0, b->cfg.by = 1, b->cfg.rows = 32;
+  }
+  const int cols = b->prec == LBM_F64           ? b->cfg.bx
+                   : b->prec == LBM_F32_SHIFT ? olbm::stream2_width(b->prec)
+                                              : 2 * olbm::batch_stream_nc(b->prec, 0);
+  long long S = 0;
+  for (const olbm::Geometry& g : b->geo) S += (long long)((g.nx + cols - 1) / cols) * g.ny;
+  auto per = [&](long long ctas) { return (S + ctas * b->sms - 1) / (ctas * b->sms); };
+  long long rows = b->prec == LBM_F64 ? per(17) : per(3);
+  if (b->prec != LBM_F64 && rows > 18) rows = std::max(12LL, per(8));
+  b->rows = (int)std::max(1LL, std::min<long long>(rows, b->cfg.rows));
+}
+
 // Rebuild the tile lists for the current launch shape.
 int build_tiles(lbm_batch* b) {
   std::vector<int4> tiles, tiles2;
   std::vector<int2> ranges, ranges2;
   if (b->cfg.kind == 1 || b->cfg.kind == 2) {
     const int nc = olbm::batch_stream_nc(b->prec, b->cfg.kind == 2 ? 0 : b->cfg.bx);
-    cut_tiles(b, 2 * nc, b->cfg.rows, tiles, ranges);
-    if (b->cfg.kind == 2) cut_tiles(b, olbm::stream2_width(b->prec), b->cfg.rows, tiles2, ranges2);
+    cut_tiles(b, 2 * nc, rows_of(b), tiles, ranges);
+    if (b->cfg.kind == 2) cut_tiles(b, olbm::stream2_width(b->prec), rows_of(b), tiles2, ranges2);
   } else {
     // kind 0: (bx or 2 bx) columns per domain, by x rows rows
     tiles.clear();
     ranges.assign(b->n, make_int2(0, 0));
     for (int k = 0; k < b->n; ++k) {
       const olbm::Geometry& g = b->geo[k];
-      const int cols = olbm::uses_pairs(b->prec, g) ? 2 * b->cfg.bx : b->cfg.bx, trows = b->cfg.by * b->cfg.rows;
+      const int cols = olbm::uses_pairs(b->prec, g) ? 2 * b->cfg.bx : b->cfg.bx, trows = b->cfg.by * rows_of(b);
       ranges[k].x = (int)tiles.size();
       for (int y0 = 0; y0 < g.ny; y0 += trows)
         for (int x0 = 0; x0 < g.nx; x0 += cols) tiles.push_back(make_int4(k, x0, y0, 0));
@@ -284,6 +316,7 @@ olbm::BatchLaunch view(const lbm_batch* b) {
   olbm::BatchLaunch v;
   v.model = b->model;
   v.cfg = b->cfg;
+  v.cfg.rows = rows_of(b);
   if (b->cfg.kind == 2) v.cfg.kind = 1, v.cfg.bx = 0;  // single steps: the kind 1 tiles
   v.desc = b->d_desc;
   v.tiles = b->d_tiles;
@@ -476,16 +509,7 @@ int lbm_batch_create(int n, const int* nx, const int* ny, const double* theta, c
     free_batch(b);
     return bfail(nullptr, LBM_ECUDA, "lbm_batch_create: %s", cudaGetErrorString(e));
   }
-  // Default tiles: FP64 the column routine with 64 x 2 threads and 16 rows; FP16
-  // the bulk-copy pipeline on tiles of 32 rows; FP32 two steps a launch on tiles of
-  // 32 rows (256 Taylor-Green domains N ~ U{64..512}, diagnostics every step: 113.3
-  // GLUPS in graph mode against 83.3 for the single-step pipeline; the persistent
-  // mode takes single steps either way).
-  if (prec == LBM_F64) {
-    b->cfg.bx = 64, b->cfg.by = 2, b->cfg.rows = 16;
-  } else {
-    b->cfg.kind = prec == LBM_F32_SHIFT ? 2 : 1, b->cfg.bx = 0, b->cfg.by = 1, b->cfg.rows = 32;
-  }
+  default_tiles(b);
   int s = build_tiles(b);
   if (s != LBM_OK) {
     char msg[320];
@@ -515,6 +539,7 @@ int lbm_batch_set_launch(lbm_batch* b, int bx, int by, int rows) {
     return bfail(b, LBM_EINVAL, "tile shape %dx%d x %d rows invalid (bx a multiple of 32, bx*by <= 512, rows 1..64)",
                  bx, by, rows);
   b->cfg = k;
+  b->rows = 0;
   return build_tiles(b);
 }
 
@@ -534,6 +559,7 @@ int lbm_batch_set_launch_ex(lbm_batch* b, int kind, int bx, int by, int rows) {
   k.by = 1;
   k.rows = rows;
   b->cfg = k;
+  b->rows = 0;
   return build_tiles(b);
 }
 
