@@ -38,19 +38,16 @@ BYTES_PER_NODE = {"f64": 144, "f32": 72, "f16": 36, "f64df": 144}
 # complete with the Eq. 12 prefactor from f^neq 82) and the fused diagnostics (5:
 # three sums and j.u by two FMAs).
 FP64_OPS_PER_NODE = {"lbgk": 60, "oreg": 93, "partial": 103, "complete": 123, "complete_neq": 120}
-# The FP64 form on GB300 is bound by the FP64 pipe, which carries only the sums and
-# FMAs of that count: the products run on the integer pipes (correctly rounded
-# binary64 products from the operands' bit fields, bit-identical to the FP64
-# instruction) and the power-of-two scalings move exponent bits there too.
-FP64_PIPE_OPS_PER_NODE = {"lbgk": 41, "oreg": 71, "partial": 73, "complete": 86, "complete_neq": 84}
-INT_PIPE_PRODUCTS_PER_NODE = {"lbgk": 17, "oreg": 20, "partial": 24, "complete": 31, "complete_neq": 29}
+# The FP64 form collides in 64-bit fixed point on the integer pipes; the FP64 pipe carries the
+# addition that rounds each of the nine results to binary64.
+FP64_PIPE_OPS_PER_NODE = 9
 FALLBACK_HBM_GBS = 6800.0
 # DRAM bytes (read + write) per node of one step-kernel launch, from ncu captures of
 # the current kernels: the FP64 kernel captured at 2048^2 and scaled to the lattice by
 # node count (its traffic grows in proportion), the FP32 kernels (single steps, and two
 # steps a launch) captured at 4096^2.
 # Keyed by (storage, model, steps per launch).
-PROFILED_TRAFFIC_B_PER_NODE = {("f64", "complete", 1): 133.7, ("f32", "complete", 1): 68.8,
+PROFILED_TRAFFIC_B_PER_NODE = {("f64", "complete", 1): 141.7, ("f32", "complete", 1): 68.8,
                                ("f32", "complete", 2): 72.1}
 MODEL_NAMES = ["lbgk", "oreg", "partial", "complete", "complete_neq"]
 # the step kernel each storage form launches under its default launch shape
@@ -293,17 +290,14 @@ def run_gpu(args):
     alu = None
     if args.prec == "f64":
         peak_ops = capi.lbm_measure_peak(0) / 2.0  # FMA instructions per second (2 FLOP each)
-        ops = FP64_PIPE_OPS_PER_NODE[args.model] * n / (step_ms * 1e-3)
+        ops = FP64_PIPE_OPS_PER_NODE * n / (step_ms * 1e-3)
         alu = {"bound": "alu", "achieved": round(ops / 1e12, 4), "peak": round(peak_ops / 1e12, 4),
-               "unit": "Top/s (FP64-pipe add/fma)", "frac": round(ops / peak_ops, 4), "traffic": traffic,
+               "unit": "Top/s (FP64-pipe additions)", "frac": round(ops / peak_ops, 4), "traffic": traffic,
                "peak_source": "FP64 FMA issue rate measured live on this GPU (lbm_measure_peak / 2)",
-               "ops_per_node": FP64_PIPE_OPS_PER_NODE[args.model],
+               "ops_per_node": FP64_PIPE_OPS_PER_NODE,
                "method_ops_per_node": FP64_OPS_PER_NODE[args.model],
-               "integer_pipe_products_per_node": INT_PIPE_PRODUCTS_PER_NODE[args.model],
                "method_ops_rate": round(FP64_OPS_PER_NODE[args.model] * n / (step_ms * 1e-3) / 1e12, 4),
                "kernel": roof["kernel"], "ms_per_launch": round(step_ms, 4)}
-        if alu["frac"] > roof["frac"]:
-            roof, alu = alu, roof
     lat.close()
     del lat
 
@@ -318,9 +312,9 @@ def run_gpu(args):
                       "l2": f"inputs larger than L2: two {lat_bytes(args.prec, n)/1e9:.2f} GB population buffers",
                       "parallelism": f"one independent lattice per GPU (replicas), {world} GPU(s)"},
            "roofline": roof, "roofline_other": alu,
-           "gpu_launches": launches * (1 + spl),
-           "gpu_launches_note": f"per launch: 1 fused step kernel ({spl} step(s)) + {spl} diagnostics finalisation "
-                                f"kernel(s)",
+           "gpu_launches": launches * 2,
+           "gpu_launches_note": f"per launch: 1 fused step kernel ({spl} step(s)) + 1 diagnostics finalisation "
+                                f"kernel",
            "clocks": clocks.summary(),
            "final_diagnostics": {"t": t_diag, "mass": diag[0], "mom_x": diag[1], "mom_y": diag[2],
                                  "kinetic": diag[3], "nonfinite": diag[4]}}
