@@ -148,7 +148,7 @@ __device__ __noinline__ void adj_node_float(const double* __restrict__ fbuf, con
 // thread, launched with programmatic serialization (plain loads after its wait). Bound by
 // the FP64 pipe before (about 210 of its operations a node, 82 % busy: 384^2 70 us a step),
 // now by the integer pipes (1024^2 gradient of 100 steps 14.2 ms with five blocks a SM, 14.5
-// with four, 14.9 with three; 384^2 12.2 -> 3.2 ms with the forward steps).
+// with four, 14.9 with three; 384^2 12.2 -> 3.3 ms with the forward steps).
 constexpr int kAFX = 64, kAFY = 2;
 #ifndef OLBM_ADJ_F64_MINB
 #define OLBM_ADJ_F64_MINB 5
