@@ -95,9 +95,9 @@ __global__ void __launch_bounds__(kTileThreads)
     const int mx = wrapx ? 0 : s, my = wrapy ? 0 : s;  // ring already consumed
     const int w = b.W - 2 * mx, h = b.H - 2 * my;
     const int cols = kF64 ? w : (w + 1) / 2;           // nodes, or node pairs, of a row
-    const unsigned inv = ((1u << 20) + (unsigned)cols - 1u) / (unsigned)cols;  // exact for idx < 2^20 / cols
+    const unsigned inv = tile_row_inv(cols);
     for (int idx = threadIdx.x; idx < cols * h; idx += blockDim.x) {
-      const int row = (int)(((unsigned long long)(unsigned)idx * inv) >> 20), col = idx - row * cols;
+      const int row = tile_row(idx, inv), col = idx - row * cols;
       const int lx = mx + (kF64 ? col : 2 * col), ly = my + row;
       int gx = b.x0 + lx, gy = b.y0 + ly;
       gx = gx < 0 ? gx + g.nx : (gx >= g.nx ? gx - g.nx : gx);

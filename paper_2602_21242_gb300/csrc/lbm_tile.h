@@ -28,6 +28,18 @@ inline long long tile_smem(const Geometry& g, int tx, int ty, int steps, int ele
   return steps < 2 ? 0 : 18LL * elem * tile_nodes(g, tx, ty, steps);
 }
 
+// Row of index idx in a region of `cols` columns, idx / cols by a multiplication (the reciprocal
+// once a step): inv = 2^28 / cols rounded up, by e < cols / 2^28 of a column too much, so the
+// quotient is exact while idx * cols < 2^28. Both are at most a region's nodes.
+__host__ __device__ inline unsigned tile_row_inv(int cols) {
+  return ((1u << 28) + (unsigned)cols - 1u) / (unsigned)cols;
+}
+__host__ __device__ inline int tile_row(int idx, unsigned inv) {
+  return (int)(((unsigned long long)(unsigned)idx * inv) >> 28);
+}
+constexpr long long kTileNodesMax = kTileSmemMax / (18 * 2);  // of the smallest storage type
+static_assert(kTileNodesMax * kTileNodesMax < (1LL << 28), "tile_row is exact for every region that fits");
+
 TilesPlan tile_plan(const Geometry& g, int prec, double theta, double tau, int sms, bool walls);
 
 cudaError_t launch_tile_f64(const StepArgs& a, const TilesPlan& p, int steps, cudaStream_t st);

@@ -1,0 +1,39 @@
+// Host check of the small-lattice tiles' index arithmetic (lbm_tile.h): for every lattice
+// width NX0 .. NX1 (step STRIDE) of NY rows that tile_plan gives a plan, the rows and
+// columns that the kernel forms from a linear index in the regions of every step of a launch, against
+// integer division, for the full tile and the ragged last ones. Prints the widths looked at,
+// those with a plan, the largest region (in columns) and the number of wrong indices.
+// Usage: tile_check PREC WALLS SMS NY NX0 NX1 STRIDE
+#include <algorithm>
+#include <cstdio>
+#include <cstdlib>
+
+#include "lbm_tile_plan.cu"
+
+using namespace olbm;
+
+int main(int, char** v) {
+  const int prec = atoi(v[1]), walls = atoi(v[2]), sms = atoi(v[3]), ny = atoi(v[4]);
+  const bool f64 = prec == 0 || prec == 3;
+  long long widths = 0, planned = 0, largest = 0, wrong = 0;
+  for (int nx = atoi(v[5]); nx <= atoi(v[6]); nx += atoi(v[7])) {
+    ++widths;
+    const Geometry g{nx, ny, nx, (long long)nx * ny};
+    const TilesPlan p = tile_plan(g, prec, 1.0 / 3.0, 0.8, sms, walls != 0);
+    if (!p.on()) continue;
+    ++planned;
+    const bool wrapx = p.tx >= nx, wrapy = p.ty >= ny;
+    const int lastx = nx - (nx - 1) / p.tx * p.tx, lasty = ny - (ny - 1) / p.ty * p.ty;
+    for (int ring = 0; ring < p.steps; ++ring)
+      for (int e = 0; e < 4; ++e) {  // full and ragged tiles
+        const int w = (e & 1 ? lastx : std::min(p.tx, nx)) + (wrapx ? 0 : 2 * ring);
+        const int h = (e & 2 ? lasty : std::min(p.ty, ny)) + (wrapy ? 0 : 2 * ring);
+        const int cols = f64 ? w : (w + 1) / 2;  // nodes, or node pairs
+        largest = std::max<long long>(largest, w);
+        const unsigned inv = tile_row_inv(cols);
+        for (int idx = 0; idx < cols * h; ++idx) wrong += tile_row(idx, inv) != idx / cols;
+      }
+  }
+  printf("%lld %lld %lld %lld\n", widths, planned, largest, wrong);
+  return 0;
+}
