@@ -154,10 +154,9 @@ constexpr int kAFX = 64, kAFY = 2;
 #define OLBM_ADJ_F64_MINB 5
 #endif
 template <int MODEL>
-__global__ void __launch_bounds__(kAFX* kAFY, OLBM_ADJ_F64_MINB) adj_step_f64_kernel(const double* __restrict__ fbuf,
-                                                                                     const double* __restrict__ lam_next,
-                                                                                     double* __restrict__ lam, Geometry g,
-                                                                                     Coef<double> c) {
+__global__ void __launch_bounds__(kAFX* kAFY, OLBM_ADJ_F64_MINB) adj_step_f64_kernel(const double* fbuf,
+                                                                                     const double* lam_next, double* lam,
+                                                                                     Geometry g, Coef<double> c) {
   const int x = blockIdx.x * kAFX + threadIdx.x, y = blockIdx.y * kAFY + threadIdx.y;
   pdl_wait();
   pdl_launch_dependents();

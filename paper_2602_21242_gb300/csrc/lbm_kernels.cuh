@@ -608,9 +608,8 @@ __global__ void __maxnreg__(OLBM_F64_MAXNREG) step_kernel_f64(const double* src,
 // take: bound by the FP64 pipe, its products on the integer pipes. Capped at 128 registers
 // (four blocks of 128 threads an SM, a few bytes spilled): 6.33 GLUPS at 4096^2.
 template <int MODEL, bool DIAG>
-__global__ void __maxnreg__(128) step_kernel_f64_float(const double* __restrict__ src, double* __restrict__ dst,
-                                                       Geometry g, Coef<double> c, double* __restrict__ partials,
-                                                       int rows) {
+__global__ void __maxnreg__(128) step_kernel_f64_float(const double* src, double* dst, Geometry g,
+                                                       Coef<double> c, double* __restrict__ partials, int rows) {
   step_body<MODEL, 0, DIAG, false>(src, dst, g, c, partials, rows);
 }
 

@@ -67,8 +67,7 @@ __device__ __noinline__ void tile_float(double* f, const Coef<CT>& c, NodeMoment
 
 template <int MODEL, int PREC, bool DIAG>
 __global__ void __launch_bounds__(kTileThreads)
-    tile_steps_kernel(const typename Form<PREC>::S* __restrict__ src, typename Form<PREC>::S* __restrict__ dst,
-                      Geometry g,
+    tile_steps_kernel(const typename Form<PREC>::S* src, typename Form<PREC>::S* dst, Geometry g,
                       Coef<typename std::conditional<kHasFixed<typename Form<PREC>::T>, typename Form<PREC>::T, f32x2>::type> c,
                       int steps, int tx, int ty, const unsigned char* __restrict__ walls,
                       double* __restrict__ partials) {
