@@ -786,8 +786,10 @@ __device__ __noinline__ void init_node_float(double r, double u, double v, const
   }
 }
 
-// The same in fixed point (lbm_fixed.cuh) for densities below 4 (shifted forms: 2) and
-// velocities below 1/2. FP64 arithmetic held this kernel on the FP64 pipe (33 operations a
+// The same in fixed point (lbm_fixed.cuh) for densities in [1/2, 4) (shifted forms: below 2)
+// and velocities below 1/2: FP64 storage keeps 2^-60 absolute there, which a lower density
+// would make a loss against binary64 (the shifted forms store deviations from the rest state of
+// density 1). FP64 arithmetic held this kernel on the FP64 pipe (33 operations a
 // node with the conversions to FP32: 1013 us in FP64 and 1279 us in FP32 at 4096^2 for
 // 96 and 60 bytes a node). The shifted forms store what the FP64 arithmetic stores, bit for
 // bit: a deviation within 2^-50 of a rounding boundary, more than either path's error
@@ -798,7 +800,8 @@ __device__ __forceinline__ void init_node(double r, double u, double v, const Fi
   constexpr bool kShift = PREC != 0;
   const unsigned rh = (unsigned)__double2hiint(r);
   const unsigned uh = (unsigned)__double2hiint(u) & 0x7FFFFFFFu, vh = (unsigned)__double2hiint(v) & 0x7FFFFFFFu;
-  bool ok = d.c.on && rh < (kShift ? 0x40000000u : 0x40100000u) && uh < 0x3FE00000u && vh < 0x3FE00000u;
+  const unsigned low = kShift ? 0u : 0x3FE00000u, high = kShift ? 0x40000000u : 0x40100000u;
+  bool ok = d.c.on && rh - low < high - low && uh < 0x3FE00000u && vh < 0x3FE00000u;
   fx::Fx<60> f[9];
   float s[9];
   if (ok) {
