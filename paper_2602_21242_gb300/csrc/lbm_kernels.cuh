@@ -862,7 +862,8 @@ __device__ __noinline__ void pulled_moments_cold(const typename Form<PREC>::S* _
 }
 
 // The sums m0, j_x, j_y of node (x, y)'s stored values, rounded to binary64, added as
-// 64-bit integers: FP64 storage with 60 fraction bits (populations below 1), the shifted
+// 64-bit integers: FP64 storage with 60 fraction bits (populations below 1, densities in
+// [1/2, 4): below 1/2 the bits dropped under 2^-60 would be a loss against binary64), the shifted
 // forms with the largest of the nine at bit 58, so that values down to 2^-35 of it are
 // exact. Left to FP64 arithmetic, the 16 additions (and nine conversions from FP32) held
 // this kernel on the FP64 pipe.
@@ -898,7 +899,8 @@ __device__ __forceinline__ void pulled_sums(const typename Form<PREC>::S* __rest
   }
   const fx::Moments m = fx::moments(a);
   if constexpr (PREC == 0) {  // (sums below 4 for the conversion)
-    ok = ok && fx::within(m.rho.v, 1 << 30) && fx::within(m.jx.v, 1 << 30) && fx::within(m.jy.v, 1 << 30);
+    const unsigned rh = (unsigned)(m.rho.v >> 32);
+    ok = ok && rh - (1u << 27) < (1u << 30) - (1u << 27) && fx::within(m.jx.v, 1 << 30) && fx::within(m.jy.v, 1 << 30);
   }
   if (!ok) {
     pulled_moments_cold<PREC>(src, g, x, y, &m0, &jx, &jy);
