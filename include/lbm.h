@@ -315,8 +315,12 @@ int lbm_run_host(lbm_ctx* ctx, const double* h_rho0, const double* h_ux0, const 
  * each thread updating `rows` nodes (node pairs for the shifted forms when nx
  * is even) of one column (1 <= rows <= 64). Results do not depend on the
  * shape except for the order of the diagnostics sums. Each storage form starts
- * from a default measured on GB300; lbm_set_launch may reallocate the small
- * diagnostics buffer (it then synchronises the stream). Errors: LBM_EINVAL.
+ * from a default measured on GB300, with which the library also runs several steps a launch
+ * on small lattices and, in FP64 storage, other rows per thread in diagnosed
+ * steps; lbm_get_launch reports the shape of its single steps. Any other shape is
+ * used as it is, for every step; setting the default shape again brings the default back
+ * with all that goes with it. lbm_set_launch may reallocate the diagnostics
+ * buffer (it then synchronises the stream). Errors: LBM_EINVAL.
  */
 int lbm_set_launch(lbm_ctx* ctx, int bx, int by, int rows);
 int lbm_get_launch(const lbm_ctx* ctx, int* bx, int* by, int* rows);
@@ -392,7 +396,9 @@ int lbm_batch_destroy(lbm_batch* b);
 
 /* Tile shape (no counterpart in the paper), launch kind 0 (the column routine): blocks of bx x by threads (bx a
  * multiple of 32, bx * by <= 512) updating tiles of bx (node pairs: 2 bx) columns x
- * by * rows rows. Rebuilds the tile list (synchronous). */
+ * by * rows rows. Rebuilds the tile list (synchronous). The default shape's rows are the most that
+ * it takes: a small batch runs fewer under it (lbm_batch_get_launch reports the shape, and in ntiles the
+ * tiles it comes to); setting that shape again is the default again, any other is used as it is. */
 int lbm_batch_set_launch(lbm_batch* b, int bx, int by, int rows);
 int lbm_batch_get_launch(const lbm_batch* b, int* bx, int* by, int* rows, int* ntiles);
 

@@ -105,6 +105,9 @@ struct lbm_batch {
   int4* d_tiles2 = nullptr;
   int2* d_ranges2 = nullptr;
   int rows = 0;  // tile rows of a small batch under the default shape (0: cfg.rows)
+  // both as lbm_batch_create chose them: lbm_batch_set_launch of that shape brings the rows back
+  olbm::LaunchCfg default_cfg;
+  int default_rows = 0;
   int ntiles2 = 0;
   double* d_parts[kParts] = {};  // per-tile partials, max(ntiles, ntiles2) each
   double* d_diag = nullptr;  // n * 5, latest fused diagnostics
@@ -216,6 +219,7 @@ void default_tiles(lbm_batch* b) {
   long long rows = b->prec == LBM_F64 ? per(17) : per(3);
   if (b->prec != LBM_F64 && rows > 18) rows = std::max(12LL, per(8));
   b->rows = (int)std::max(1LL, std::min<long long>(rows, b->cfg.rows));
+  b->default_cfg = b->cfg, b->default_rows = b->rows;
 }
 
 // Rebuild the tile lists for the current launch shape.
@@ -539,7 +543,7 @@ int lbm_batch_set_launch(lbm_batch* b, int bx, int by, int rows) {
     return bfail(b, LBM_EINVAL, "tile shape %dx%d x %d rows invalid (bx a multiple of 32, bx*by <= 512, rows 1..64)",
                  bx, by, rows);
   b->cfg = k;
-  b->rows = 0;
+  b->rows = olbm::same_shape(k, b->default_cfg) ? b->default_rows : 0;
   return build_tiles(b);
 }
 
@@ -559,7 +563,7 @@ int lbm_batch_set_launch_ex(lbm_batch* b, int kind, int bx, int by, int rows) {
   k.by = 1;
   k.rows = rows;
   b->cfg = k;
-  b->rows = 0;
+  b->rows = olbm::same_shape(k, b->default_cfg) ? b->default_rows : 0;
   return build_tiles(b);
 }
 

@@ -258,6 +258,9 @@ int lbm_create_ex(int nx, int ny, double theta, double tau, int model, int prec,
   // whose last bits differ from the node pairs of the tiles: they keep single steps.
   if (c->cfg.kind != 0 || prec == LBM_F64 || prec == LBM_F64_DF || nx % 2 == 0)
     for (int w = 0; w < 2; ++w) c->tile[w] = olbm::tile_plan(c->g, prec, theta, tau, sms, w != 0);
+  c->default_cfg = c->cfg;
+  c->default_diag_rows = c->diag_rows;
+  for (int w = 0; w < 2; ++w) c->default_tile[w] = c->tile[w];
   // (a cut into tiles has at most two an SM)
   // (diagnosed steps take at least as many rows, so no more partials, unless one row is all there is)
   c->parts_cap = std::max(c->nparts, 2LL * sms);
@@ -396,7 +399,7 @@ int lbm_set_walls(lbm_ctx* ctx, const unsigned char* h_mask, long long* h_count)
     if (e == cudaSuccess)
       e = cudaMemcpy(ctx->d_walls, list, sizeof(int2) * (size_t)n, cudaMemcpyHostToDevice);
     delete[] list;
-    if (e == cudaSuccess && ctx->tile[1].on()) {
+    if (e == cudaSuccess && ctx->default_tile[1].on()) {  // (whatever lbm_set_launch chose or will choose)
       e = cudaMalloc(&ctx->d_wall_mask, (size_t)nodes);
       if (e == cudaSuccess) e = cudaMemcpy(ctx->d_wall_mask, h_mask, (size_t)nodes, cudaMemcpyHostToDevice);
     }
@@ -756,9 +759,11 @@ int lbm_set_launch_ex(lbm_ctx* ctx, int kind, int bx, int by, int rows) {
     ctx->parts_total = total;
     ctx->parts_cap = need;
   }
-  ctx->cfg = k;
-  ctx->diag_rows = 0;
-  ctx->tile[0] = ctx->tile[1] = olbm::TilesPlan{};  // the chosen shape, nothing else
+  // the default shape brings back all that goes with it; any other is the chosen shape and nothing else
+  const bool dflt = olbm::same_shape(k, ctx->default_cfg);
+  ctx->cfg = dflt ? ctx->default_cfg : k;
+  ctx->diag_rows = dflt ? ctx->default_diag_rows : 0;
+  for (int w = 0; w < 2; ++w) ctx->tile[w] = dflt ? ctx->default_tile[w] : olbm::TilesPlan{};
   ctx->nparts = need;
   return LBM_OK;
 }

@@ -20,8 +20,13 @@ struct lbm_ctx {
   cudaStream_t stream = nullptr;
   olbm::LaunchCfg cfg{};
   int diag_rows = 0;  // rows of a diagnosed step under the default FP64 launch (0: as cfg)
-  // several steps a launch on small lattices, without and with walls; off once lbm_set_launch chose a shape
+  // several steps a launch on small lattices, without and with walls; off while lbm_set_launch's shape is another
+  // than the default one
   olbm::TilesPlan tile[2]{};
+  // the three as lbm_create chose them: lbm_set_launch of that shape brings them back
+  olbm::LaunchCfg default_cfg{};
+  int default_diag_rows = 0;
+  olbm::TilesPlan default_tile[2]{};
   // Per-block diagnostics partials: kGroups groups of olbm::kFinalJobs buffers of parts_cap
   // blocks each, in one allocation (its start also serves lbm_diagnostics). Diagnosed steps
   // fill a group's buffers in turn; the final sums of a full group are one launch on a second
@@ -59,7 +64,7 @@ struct lbm_ctx {
   // fullway bounce-back wall nodes (x, y), applied after every step (lbm_set_walls)
   int2* d_walls = nullptr;
   long long n_walls = 0;
-  unsigned char* d_wall_mask = nullptr;  // nx * ny bytes, where tile[1] is used and walls are set
+  unsigned char* d_wall_mask = nullptr;  // nx * ny bytes, where default_tile[1] is used and walls are set
   // Slab halo trade (lbm_halo_pack / lbm_halo_unpack): the time of the last
   // unpack, or of lbm_init / lbm_set_state (a pack needs exactly one step
   // since), and the time of the last pack (an unpack needs one at this time).

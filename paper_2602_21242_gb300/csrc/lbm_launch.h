@@ -30,6 +30,11 @@ inline bool valid_cfg(const LaunchCfg& k) {
          k.rows <= 64;
 }
 
+// The same launch (kinds 1 and 2 do not use by).
+inline bool same_shape(const LaunchCfg& a, const LaunchCfg& b) {
+  return a.kind == b.kind && a.bx == b.bx && a.rows == b.rows && (a.kind != 0 || a.by == b.by);
+}
+
 struct StepArgs {
   int model;         // 0..3, enum lbm_model
   bool diag;         // fuse the diagnostics reduction into this step
