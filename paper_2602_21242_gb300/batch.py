@@ -27,6 +27,7 @@ class Batch:
         with torch.cuda.device(self.device):
             self._b = capi.lbm_batch_create(self.nx, self.ny, self.theta, self.tau, self.model, self.prec,
                                             self.stream.cuda_stream)
+        self.default_launch = self.launch()[:4]
         self.set_mode(mode)
 
     @property

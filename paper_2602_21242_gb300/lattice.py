@@ -50,6 +50,8 @@ class Lattice:
                 ptr = self._buffers.data_ptr()
             self._ctx = capi.lbm_create_ex(self.nx, self.ny, self.theta, self.tau, self.model, self.prec,
                                            self.stream.cuda_stream, ptr)
+        self.default_launch = capi.lbm_get_launch_ex(self._ctx)
+        self._walls = None
 
     # -- lifecycle
     def close(self) -> None:
@@ -133,7 +135,10 @@ class Lattice:
             if tuple(np.shape(mask)) != (self.ny, self.nx):
                 raise ValueError(f"wall mask must have shape {(self.ny, self.nx)}")
         with torch.cuda.device(self.device):
-            return capi.lbm_set_walls(self._ctx, mask)
+            self._walls = None
+            count = capi.lbm_set_walls(self._ctx, mask)
+            self._walls = mask if count else None
+            return count
 
     def step_diagnostics(self, raise_nonfinite: bool = True):
         with torch.cuda.device(self.device):

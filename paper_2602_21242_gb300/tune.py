@@ -1,9 +1,11 @@
 """Autotuner for the launch shape of the step kernels.
 
-For a lattice (or a batch) it times candidate shapes (threads bx x by, rows per
-thread) with CUDA events on the object's own stream, keeps the fastest, and
+For a lattice (or a batch) it times the default launch and candidate shapes (threads bx x by,
+rows per thread) with CUDA events on the object's own stream, keeps the fastest, and
 caches it in a JSON file keyed by GPU name, kind, size class, storage form and
-collision model, so the measurement runs once per configuration class.
+collision model, so the measurement runs once per configuration class. The default is more than
+a shape (several steps a launch on small lattices, rows that depend on the size), so it is
+kept, and cached, as the default.
 
 Cache file: $OLBM_TUNE_CACHE, else ~/.cache/olbm/tune.json.
 """
@@ -63,7 +65,8 @@ def _store(path: str, key: str, value) -> None:
 def _key(kind: str, nodes: int, prec: int, model: int, extra: str = "") -> str:
     gpu = torch.cuda.get_device_name(torch.cuda.current_device()).replace(" ", "_")
     size_class = int(round(math.log2(max(nodes, 1))))
-    return f"{gpu}|{kind}|2^{size_class}{extra}|prec{prec}|model{model}"
+    # (|d: the default launch was among the candidates; entries of other keys were chosen without it)
+    return f"{gpu}|{kind}|2^{size_class}{extra}|prec{prec}|model{model}|d"
 
 
 def _timing_fields(nx: int, ny: int):
@@ -75,38 +78,50 @@ def _timing_fields(nx: int, ny: int):
 
 def _time(step, sync, stream, steps: int) -> float:
     step(steps)  # warm-up with the same count (a batch captures its graph here)
-    sync()
-    e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-    e0.record(stream)
-    step(steps)
-    e1.record(stream)
-    sync()
-    return e0.elapsed_time(e1) / steps
+    best = math.inf
+    for _ in range(3):
+        sync()
+        e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        e0.record(stream)
+        step(steps)
+        e1.record(stream)
+        sync()
+        best = min(best, e0.elapsed_time(e1) / steps)
+    return best
 
 
 def tune_lattice(lat, candidates=None, steps: int = 10, use_cache: bool = True, path: str | None = None):
     """Pick and apply the fastest launch (kind, bx, by, rows) for `lat` (a Lattice). Timing
     runs on a temporary lattice of the same size, storage and model started from the
     advected shear wave of `_timing_fields`, so `lat`'s state is untouched. Candidates may
-    be given as (bx, by, rows) for kind 0 or as (kind, bx, by, rows). Returns ((kind, bx, by, rows), ms_per_step or None if cached)."""
+    be given as (bx, by, rows) for kind 0 or as (kind, bx, by, rows); otherwise the default launch
+    is the first, and another replaces it only if it is faster with diagnostics every step
+    and not slower (by more than the timing's 2 %) without. `lat`'s walls are those it has now. Returns
+    ((kind, bx, by, rows), ms_per_step or None if cached)."""
     from .lattice import Lattice
 
     path = path or cache_path()
-    key = _key("lattice", lat.nx * lat.ny, lat.prec, lat.model, f"|nx={lat.nx}")
+    walls = lat._walls
+    key = _key("lattice", lat.nx * lat.ny, lat.prec, lat.model, f"|nx={lat.nx}" + ("|walls" if walls is not None else ""))
     if use_cache:
         hit = _load_cache(path).get(key)
         if hit:
-            capi.lbm_set_launch_ex(lat.ctx, *hit["shape"])
-            return tuple(hit["shape"]), None
-    if candidates is None:
-        candidates = list(LATTICE_CANDIDATES)
+            shape = lat.default_launch if hit.get("default") else tuple(hit["shape"])
+            capi.lbm_set_launch_ex(lat.ctx, *shape)
+            return shape, None
+    keep_default = candidates is None
+    if keep_default:
+        candidates = [lat.default_launch] + LATTICE_CANDIDATES
         if lat.prec != capi.LBM_F64_DF:  # shapes a form does not take are skipped below
             candidates += PIPELINE_CANDIDATES + TWO_STEP_CANDIDATES
     best = None
     with Lattice(lat.nx, lat.ny, lat.theta, lat.tau, lat.model, lat.prec, device=lat.device,
                  stream=lat.stream) as tmp:
         tmp.init(*(torch.from_numpy(a).to(lat.device) for a in _timing_fields(lat.nx, lat.ny)))
+        if walls is not None:
+            tmp.set_walls(walls)
         tmp.set_diagnostics_interval(1)
+        plain_default = math.inf
         for shape in candidates:
             shape = tuple(shape) if len(shape) == 4 else (0,) + tuple(shape)
             try:
@@ -114,10 +129,19 @@ def tune_lattice(lat, candidates=None, steps: int = 10, use_cache: bool = True, 
             except capi.LBMError:
                 continue
             ms = _time(tmp.step, tmp.sync, tmp.stream, steps)
-            if best is None or ms < best[1]:
-                best = (shape, ms)
+            if best is not None and ms >= best[1]:
+                continue
+            if keep_default:
+                tmp.set_diagnostics_interval(0)
+                plain = _time(tmp.step, tmp.sync, tmp.stream, steps)
+                tmp.set_diagnostics_interval(1)
+                if best is None:
+                    plain_default = plain
+                elif plain > 1.02 * plain_default:
+                    continue
+            best = (shape, ms)
     capi.lbm_set_launch_ex(lat.ctx, *best[0])
-    _store(path, key, {"shape": list(best[0]), "ms_per_step": best[1]})
+    _store(path, key, {"shape": list(best[0]), "ms_per_step": best[1], "default": best[0] == lat.default_launch})
     return tuple(best[0]), best[1]
 
 
@@ -125,20 +149,21 @@ def tune_batch(batch, candidates=None, steps: int = 10, use_cache: bool = True, 
     """Pick and apply the fastest tile shape for `batch` (a Batch). The timing steps the
     batch itself from the advected shear wave of `_timing_fields`: call it before Batch.init.
     Candidates are (kind, bx, by, rows) or (bx, by, rows) for kind 0; the default set
-    adds the pipeline shapes for the shifted forms. Returns ((kind, bx, by, rows),
+    begins with the batch's default launch and adds the pipeline shapes for the shifted forms. Returns ((kind, bx, by, rows),
     ms_per_step or None if cached)."""
     path = path or cache_path()
     key = _key("batch", batch.total_nodes, batch.prec, batch.model, f"|n{batch.n}|k")
     if use_cache:
         hit = _load_cache(path).get(key)
         if hit:
-            batch.set_launch(*hit["shape"])
-            return tuple(hit["shape"]), None
+            shape = batch.default_launch if hit.get("default") else tuple(hit["shape"])
+            batch.set_launch(*shape)
+            return shape, None
     rho, ux, uy = zip(*(_timing_fields(nx, ny) for nx, ny in zip(batch.nx, batch.ny)))
     best = None
     if candidates is None:
-        candidates = BATCH_CANDIDATES + (BATCH_PIPELINE_CANDIDATES + BATCH_TWO_STEP_CANDIDATES
-                                         if batch.prec != capi.LBM_F64 else [])
+        candidates = [batch.default_launch] + BATCH_CANDIDATES + (
+            BATCH_PIPELINE_CANDIDATES + BATCH_TWO_STEP_CANDIDATES if batch.prec != capi.LBM_F64 else [])
     for shape in candidates:
         shape = tuple(shape) if len(shape) == 4 else (0,) + tuple(shape)
         try:
@@ -151,5 +176,5 @@ def tune_batch(batch, candidates=None, steps: int = 10, use_cache: bool = True, 
             best = (shape, ms)
     batch.set_launch(*best[0])
     batch.init(rho, ux, uy)
-    _store(path, key, {"shape": list(best[0]), "ms_per_step": best[1]})
+    _store(path, key, {"shape": list(best[0]), "ms_per_step": best[1], "default": best[0] == batch.default_launch})
     return tuple(best[0]), best[1]
