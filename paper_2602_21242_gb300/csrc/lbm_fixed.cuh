@@ -153,10 +153,41 @@ struct Coefs {
   int on;              // theta in the range of the formats
 };
 
-// x to the nearest 2^-F, |x| < 2^(63 - F); in extended precision, so that no coefficient is
-// rounded to binary64 on its way.
-template <int F> inline Fx<F> fx_of(long double x) {
-  return Fx<F>{(i64)__builtin_llrintl(x * ((long double)(1ull << (F - 30)) * (1ull << 30)))};
+// A sum h + l of two binary64, |l| at most half an ulp of h: about 104 bits, for the
+// coefficients, which no rounding to binary64 shall touch on their way. (Not long double: on Arm
+// that is software, 0.67 us for the coefficients of one launch (0.09 so) where the launch of a small
+// lattice takes 4.5 us of host time; on x86 it has 64 bits.) Products are written
+// as fma(a, b, 0) so that the compiler contracts none of them with an addition.
+struct Wide {
+  double h, l;
+};
+inline Wide wide_sum(double a, double b) {  // exact
+  const double s = a + b, z = s - a;
+  return Wide{s, (a - (s - z)) + (b - z)};
+}
+inline Wide operator+(Wide a, Wide b) {
+  const Wide s = wide_sum(a.h, b.h);
+  return wide_sum(s.h, s.l + (a.l + b.l));
+}
+inline Wide operator-(Wide a, Wide b) { return a + Wide{-b.h, -b.l}; }
+inline Wide operator*(Wide a, Wide b) {
+  const double p = __builtin_fma(a.h, b.h, 0.0);
+  return wide_sum(p, __builtin_fma(a.h, b.h, -p) + __builtin_fma(a.h, b.l, __builtin_fma(a.l, b.h, 0.0)));
+}
+inline Wide operator/(Wide a, Wide b) {  // two corrections of the quotient of the leading parts
+  const double q = a.h / b.h;
+  const Wide r = a - b * Wide{q, 0.0};
+  const double q1 = r.h / b.h;
+  const Wide r1 = r - b * Wide{q1, 0.0};
+  return wide_sum(q, q1) + Wide{r1.h / b.h, 0.0};
+}
+
+// x to the nearest 2^-F, |x| < 2^(63 - F).
+template <int F> inline Fx<F> fx_of(Wide x) {
+  const double scale = (double)(1ull << (F - 30)) * (double)(1ull << 30);  // 2^F: exact products
+  const double t = __builtin_fma(x.h, scale, 0.0);
+  const i64 h = (i64)__builtin_llrint(t);
+  return Fx<F>{h + (i64)__builtin_llrint((t - (double)h) + __builtin_fma(x.l, scale, 0.0))};
 }
 
 inline Coefs make_coefs(double theta, double tau) {
@@ -164,19 +195,21 @@ inline Coefs make_coefs(double theta, double tau) {
   memset(&c, 0, sizeof c);
   c.on = theta >= 0.21 && theta <= 0.65 && tau <= 1e9 ? 1 : 0;  // omega' < 1 with 63 fraction bits
   if (!c.on) return c;
-  const long double th = theta, omp = 1.0L - 1.0L / tau;
-  c.k1 = op(fx_of<60>(omp / (4.0L * th * th)));
+  const Wide one{1.0, 0.0}, two{2.0, 0.0}, three{3.0, 0.0}, four{4.0, 0.0}, th{theta, 0.0};
+  const Wide omp = one - one / Wide{tau, 0.0}, th2 = th * th, rest = one - th, c3 = one - three * th;
+  const Wide inv = one / th, q2 = one / (four * th2);
+  c.k1 = op(fx_of<60>(omp * q2));
   c.theta_op = op(fx_of<63>(th));
   c.omp = op(fx_of<63>(omp));
-  c.q2 = op(fx_of<60>(1.0L / (4.0L * th * th)));
-  c.inv_theta = op(fx_of<60>(1.0L / th));
-  c.e2 = op(fx_of<61>((1.0L - th) / (2.0L * th)));
+  c.q2 = op(fx_of<60>(q2));
+  c.inv_theta = op(fx_of<60>(inv));
+  c.e2 = op(fx_of<61>(rest * inv / two));
   c.theta = fx_of<62>(th);
-  c.h = fx_of<62>(th * (1.0L - th));
-  c.t = fx_of<62>(th * (1.0L - 3.0L * th));
-  c.c3 = fx_of<62>(1.0L - 3.0L * th);
-  c.v0 = fx_of<60>((1.0L - th) / th);
-  c.theta2 = fx_of<60>(th * th);
+  c.h = fx_of<62>(th * rest);
+  c.t = fx_of<62>(th * c3);
+  c.c3 = fx_of<62>(c3);
+  c.v0 = fx_of<60>(rest * inv);
+  c.theta2 = fx_of<60>(th2);
   return c;
 }
 
