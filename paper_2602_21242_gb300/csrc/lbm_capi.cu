@@ -568,6 +568,10 @@ int lbm_step(lbm_ctx* ctx, int n) {
     const int done = many > 1 ? many : (two ? 2 : 1);
     ctx->t += done;
     k += done;
+    // The final sum of the call's last diagnosed steps beside the steps that follow them.
+    if (jobs.count > 0 && k < n && ctx->diag_every - (ctx->t - 1) % ctx->diag_every > n - k &&
+        (e = sum_group(false)) != cudaSuccess)
+      return cuda_fail(ctx, e, "lbm_step diagnostics launch");
   }
   cudaError_t e = sum_group(true);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "lbm_step diagnostics launch");

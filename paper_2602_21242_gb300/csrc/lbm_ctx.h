@@ -29,9 +29,10 @@ struct lbm_ctx {
   olbm::TilesPlan default_tile[2]{};
   // Per-block diagnostics partials: kGroups groups of olbm::kFinalJobs buffers of parts_cap
   // blocks each, in one allocation (its start also serves lbm_diagnostics). Diagnosed steps
-  // fill a group's buffers in turn; the final sums of a full group are one launch on a second
-  // stream, while later steps fill the other group, and lbm_step joins that stream back
-  // into `stream` before it returns (a call that fills no group sums on `stream` itself).
+  // fill a group's buffers in turn; the final sums of a group that is full, or that the last diagnosed
+  // step of a call ends before its last step, are one launch on a second stream, while later
+  // steps run, and lbm_step joins that stream back into `stream` before it returns (a call
+  // without such a group sums on `stream` itself).
   static constexpr int kGroups = 2;
   double* d_parts = nullptr;
   double* parts(int group, int k) const { return d_parts + 5 * parts_cap * (group * olbm::kFinalJobs + k); }

@@ -48,7 +48,10 @@ int stream_ctas_per_sm(int) { return OLBM_STREAM_CTAS; }
 // A sum alone is a launch, two events and a stream wait for the host and breaks the chain of
 // programmatically launched steps; on small lattices that was most of a diagnosed step
 // (64^2, diagnostics every step: FP32 10.9 -> 3.8 us, FP64 10.9 -> 5.3).
-constexpr int kFinalThreads = 512;
+// 128 threads: the butterfly of every warp goes through the FP64 pipe of one SM, which holds it longer
+// than more threads save at any number of partials (a call of one diagnosed step with its sum, us, by
+// threads 128 / 256 / 512: 64^2 FP32 8.3 / 10.3 / 12.4, 1024^2 FP16 20.6 / 20.6 / 23.6).
+constexpr int kFinalThreads = 128;
 __global__ void __launch_bounds__(kFinalThreads) finalize_kernel(FinalJobs jobs, double rho_ref, long long nodes,
                                                                  double* __restrict__ out,
                                                                  unsigned long long* __restrict__ sticky) {
