@@ -27,15 +27,16 @@ struct lbm_ctx {
   olbm::LaunchCfg default_cfg{};
   int default_diag_rows = 0;
   olbm::TilesPlan default_tile[2]{};
-  // Per-block diagnostics partials: kGroups groups of olbm::kFinalJobs buffers of parts_cap
+  // Per-block diagnostics partials: kGroups groups of group_jobs buffers of parts_cap
   // blocks each, in one allocation (its start also serves lbm_diagnostics). Diagnosed steps
   // fill a group's buffers in turn; the final sums of a group that is full, or that the last diagnosed
   // step of a call ends before its last step, are one launch on a second stream, while later
   // steps run, and lbm_step joins that stream back into `stream` before it returns (a call
   // without such a group sums on `stream` itself).
   static constexpr int kGroups = 2;
+  int group_jobs = olbm::kFinalJobs;
   double* d_parts = nullptr;
-  double* parts(int group, int k) const { return d_parts + 5 * parts_cap * (group * olbm::kFinalJobs + k); }
+  double* parts(int group, int k) const { return d_parts + 5 * parts_cap * (group * group_jobs + k); }
   long long nparts = 0;       // partials the step kernel writes under cfg
   long long parts_cap = 0;    // partials of one buffer
   long long parts_total = 0;  // partials allocated
