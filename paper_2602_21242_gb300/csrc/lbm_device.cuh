@@ -659,16 +659,20 @@ __device__ __forceinline__ bool to_fixed(const double (&f)[9], fx::Fx<60> (&a)[9
 // Collision of one FP64 node in fixed point (lbm_fixed.cuh); false for a node outside its
 // range, for which nothing is stored: that is a property of the node alone. next(f) is called
 // as soon as f is free and may load the next node's populations into it; sink receives the
-// node's FixedMoments and store(i, v) each post-collision population.
+// node's FixedMoments and store(i, v) each post-collision population. *none (if not null) is set
+// where no node of the warp has its moments in range.
 template <int MODEL, typename Sink, typename Next, typename Store>
 __device__ __forceinline__ bool collide_fixed(double (&f)[9], const fx::Coefs& c, Sink&& sink, Next&& next,
-                                              Store&& store) {
+                                              Store&& store, bool* none = nullptr) {
   fx::Fx<60> a[9], o[9];
   bool ok = to_fixed(f, a);
   next(f);
   const fx::Moments m = fx::moments(a);
   ok = ok && fx::moments_in_range(m.rho, m.jx, m.jy);
-  if (!__any_sync(__activemask(), ok)) return false;
+  if (!__any_sync(__activemask(), ok)) {
+    if (none) *none = true;
+    return false;
+  }
   fx::Fx<60> ke2;
   ok = ok && fx::collide<MODEL>(m, a, c, o, ke2);
   if (ok) {

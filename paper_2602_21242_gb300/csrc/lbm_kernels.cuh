@@ -191,11 +191,12 @@ template <typename CT> struct DiagAcc {
 struct Sum96 {
   unsigned lo = 0, mid = 0;
   int hi = 0;
-  __device__ __forceinline__ void add(long long v) {
+  __device__ __forceinline__ void add(unsigned l, unsigned m, int h) {
     asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.s32 %2, %2, %5;"
         : "+r"(lo), "+r"(mid), "+r"(hi)
-        : "r"((unsigned)v), "r"((unsigned)(v >> 32)), "r"((int)(v >> 63)));
+        : "r"(l), "r"(m), "r"(h));
   }
+  __device__ __forceinline__ void add(long long v) { add((unsigned)v, (unsigned)(v >> 32), (int)(v >> 63)); }
 };
 struct FixedDiagAcc {
   Sum96 s[4];
@@ -204,6 +205,10 @@ struct FixedDiagAcc {
     s[1].add(m.jx);
     s[2].add(m.jy);
     s[3].add(m.ke2);
+  }
+  __device__ __forceinline__ void add(const FixedDiagAcc& o) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) s[k].add(o.s[k].lo, o.s[k].mid, o.s[k].hi);
   }
 };
 // The same over a block, with the accumulators v and bad of the nodes outside the fixed-point
@@ -373,14 +378,15 @@ template <int MODEL, int PREC, bool DIAG, bool PAIRS, bool CG = false> struct Co
     }
   }
 
-  // FP64 storage, the form's own arithmetic: the rows r of the column with bit r of
-  // `left` set. Out of line: the rows that the fixed-point collision leaves out are rare,
-  // and its registers would burden the loop that handles the others. The next row's
+  // FP64 storage: the rows r of the column with bit r of `left` set, which the fixed-point loop left out:
+  // nodes outside its range in the form's own arithmetic, the others in fixed point (the loop
+  // ends at the first row that has none in range, and later rows may). Out of line: these rows
+  // are rare, and the registers would burden the loop that handles the others. The next row's
   // loads are in flight during the current row's arithmetic (in the double-word form in
   // the registers of the row just split).
-  __device__ static __noinline__ void run_float(const S* __restrict__ src, S* __restrict__ dst, const Geometry& g,
-                                                const Coef<CT>& c, int x, int xm, int xp, int y0, int dy, int rows,
-                                                unsigned long long left, DiagAcc<CT>& acc) {
+  __device__ static __noinline__ void run_rest(const S* src, S* dst, const Geometry& g, const Coef<CT>& c, int x,
+                                               int xm, int xp, int y0, int dy, int rows, unsigned long long left,
+                                               DiagAcc<CT>& acc, FixedDiagAcc& facc) {
     using Raw = Column<MODEL, 0, DIAG, false, CG>;
     int mode = 0;  // FP64: which products this warp's nodes take (see collide)
     const unsigned warp = __activemask();
@@ -396,27 +402,56 @@ template <int MODEL, int PREC, bool DIAG, bool PAIRS, bool CG = false> struct Co
         auto sink = [&](const NodeMoments<CT>& m) {
           if constexpr (DIAG) acc.add(m);
         };
+        auto store = [&](int i, double v) { q[i * g.plane] = v; };
+        auto in_fixed = [&](double (&h)[9]) {
+          return collide_fixed<MODEL>(
+              h, c.fixed,
+              [&](const FixedMoments& m) {
+                if constexpr (DIAG) facc.add(m);
+              },
+              [](double (&)[9]) {}, store);
+        };
         if constexpr (PREC == 3) {
           df64 d[9];
           split_node(f, d);
+          // The leading words tell most nodes outside the range (their sums err by less than 1e-5 where every
+          // population is below 1): a few FP32 operations in place of the integer conversions.
+          const float d13 = d[1].hi - d[3].hi, d24 = d[2].hi - d[4].hi, d57 = d[5].hi - d[7].hi, d68 = d[6].hi - d[8].hi;
+          const float rho = d[0].hi + ((d[1].hi + d[3].hi) + (d[2].hi + d[4].hi)) +
+                            ((d[5].hi + d[7].hi) + (d[6].hi + d[8].hi));
+          const float jmax = 0.501f * rho;
+          bool done = rho > 0.499f && rho < 4.001f && fabsf(d13 + (d57 - d68)) < jmax && fabsf(d24 + (d57 + d68)) < jmax;
+          if (done) done = in_fixed(f);
           if (loaded) Raw::pull(src, g, x, xm, xp, y + dy, f);
-          collide_df<MODEL>(d, c, sink, [&](int i, df64 v) {
-            q[i * g.plane] = kDfJoin == 2 ? join_f64_int(v) : (kDfJoin == 1 ? join_f64_fp64pipe(v) : join_f64(v));
-          });
+          if (!done)
+            collide_df<MODEL>(d, c, sink, [&](int i, df64 v) {
+              store(i, kDfJoin == 2 ? join_f64_int(v) : (kDfJoin == 1 ? join_f64_fp64pipe(v) : join_f64(v)));
+            });
         } else if constexpr (PREC == 0) {
-          double fn[9];
+          double fn[9], h[9];
           if (loaded) Raw::pull(src, g, x, xm, xp, y + dy, fn);
-          collide<MODEL, false, double>(
-              f, c, sink, [&](double (&h)[9]) { Raw::pull(src, g, x, xm, xp, y, h); }, &mode);
 #pragma unroll
-          for (int i = 0; i < 9; ++i) q[i * g.plane] = f[i], f[i] = fn[i];
+          for (int i = 0; i < 9; ++i) h[i] = f[i];
+          if (!in_fixed(h)) {
+            collide<MODEL, false, double>(
+                f, c, sink, [&](double (&h)[9]) { Raw::pull(src, g, x, xm, xp, y, h); }, &mode);
+#pragma unroll
+            for (int i = 0; i < 9; ++i) store(i, f[i]);
+          }
+#pragma unroll
+          for (int i = 0; i < 9; ++i) f[i] = fn[i];
         }
       }
       __syncwarp(warp);
     }
   }
 
-  // FP64 storage: the rows of a column in fixed point; returns the rows it left out. Byte
+  // FP64 storage: the rows of a column in fixed point; returns the rows it left out, which are
+  // all rows from the first one on that has no node of the warp in range. (In a flow of another unit of
+  // density, or faster than 1/2, that is the first: us a step at 4096^2, density 10, with every row tried first -> now,
+  // and with every node in the form's own arithmetic inline: FP64 2751 -> 2714, 2474; double-word 889 -> 787,
+  // 624. Those rows inline here as well would take that to 2518 and 657, but slow the rows in range down by
+  // 2 to 3 % through their registers.) Byte
   // offsets inside a plane as OFF: 32 bits where a plane is below 4 GiB, so that the nine
   // loads and stores of a node take a uniform base and one 32-bit offset each instead of a
   // 64-bit address (CG: for data written earlier in the same launch).
@@ -442,6 +477,7 @@ template <int MODEL, int PREC, bool DIAG, bool PAIRS, bool CG = false> struct Co
     if (y < g.ny) load(y, f);
     for (int r = 0; r < rows && y < g.ny; ++r, y += dy) {
       const OFF q = (OFF)y * pitch + (OFF)x * 8;
+      bool none = false;
       const bool done = collide_fixed<MODEL>(
           f, c,
           [&](const FixedMoments& m) {
@@ -452,8 +488,10 @@ template <int MODEL, int PREC, bool DIAG, bool PAIRS, bool CG = false> struct Co
           },
           [&](int i, double v) {
             *reinterpret_cast<double*>(reinterpret_cast<char*>(dst + i * g.plane) + q) = v;
-          });
+          },
+          &none);
       left |= done ? 0ull : 1ull << r;
+      if (none) return left | ~0ull << r;
     }
     return left;
   }
@@ -480,12 +518,12 @@ template <int MODEL, int PREC, bool DIAG, bool PAIRS, bool CG = false> struct Co
           g.plane < (1LL << 29) ? run_fixed<unsigned>(src, dst, g, c.fixed, x, xm, xp, y0, dy, rows, facc)
                                 : run_fixed<unsigned long long>(src, dst, g, c.fixed, x, xm, xp, y0, dy, rows, facc);
       if (__any_sync(__activemask(), left != 0)) {
-        DiagAcc<CT> rest;  // (acc itself stays in registers: its address goes nowhere)
-        run_float(src, dst, g, c, x, xm, xp, y0, dy, rows, left, rest);
+        DiagAcc<CT> rest;  // (acc and facc themselves stay in registers: their addresses go nowhere)
+        FixedDiagAcc frest;
+        run_rest(src, dst, g, c, x, xm, xp, y0, dy, rows, left, rest, frest);
         if constexpr (DIAG) {
-#pragma unroll
-          for (int k = 0; k < 4; ++k) acc.v[k] += rest.v[k];
-          acc.bad += rest.bad;
+          acc = rest;  // (nothing else adds to it)
+          facc.add(frest);
         }
       }
       return;
