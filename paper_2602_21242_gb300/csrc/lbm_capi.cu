@@ -102,13 +102,14 @@ olbm::LaunchCfg default_cfg(int prec, const olbm::Geometry& g, int sms) {
     olbm::LaunchCfg k2 = k;
     k2.kind = 2, k2.bx = 0, k2.rows = g.nx >= 8192 && g.ny >= 8192 ? 48 : 24;
     if (olbm::uses_step2(prec, g, k2)) {
-      // Smaller lattices (four CTAs an SM resident): the rows that make one wave while those
-      // are few, else those that make at least two (us a step: 512^2 3 rows 5.1, 1 row 7.4;
-      // 768^2 6 rows 7.8, 3 rows 8.6; 1536^2 8 rows 21.7, 16 rows 23.5; 2048^2 12 to 16 rows
-      // 33.2 to 33.6, 24 rows 37.6).
+      // Smaller lattices (four CTAs an SM resident): the rows that make one wave, up to 24, or, up to
+      // 40 rows of strips a resident CTA, two. us a step: 512^2 3 rows 5.1, 1 row 7.4; 768^2 6
+      // rows 7.8, 3 rows 8.6; 1200^2 10 rows (one wave) 12.3, 6 rows 13.5, 4 rows (the third wave part-filled)
+      // 14.4; 1800^2 24 rows (one wave) 26.3, 12 rows 26.7, 11 rows 28.0; 2048^2 16 rows 33.5, 24 rows
+      // 37.8; 3467 x 1744 24 rows 45.7, 21 rows (two waves) 47.2.
       const long long wave = 4LL * sms, strips = (g.nx + olbm::step2_tile_width(prec) - 1) / olbm::step2_tile_width(prec);
-      const long long one = (strips * g.ny + wave - 1) / wave, two = strips * g.ny / (2 * wave);
-      k2.rows = (int)std::max<long long>(1, std::min<long long>(k2.rows, one <= 9 ? one : two));
+      const long long work = strips * g.ny, rows = (work + wave - 1) / wave;
+      if (rows <= 40) k2.rows = (int)(rows <= 24 ? rows : (work + 2 * wave - 1) / (2 * wave));
       return k2;
     }
     k.bx = 64, k.rows = k.rows < 4 ? k.rows : 4;

@@ -1,0 +1,25 @@
+"""Rows of the FP32 form's default launch: not slower than the shapes that the default took before rows were
+chosen by waves. Margin: 3 %, what repeated timings differ by at most (the faults were 7 to 16 %)."""
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from paper_2602_21242_gb300 import capi, flows
+from paper_2602_21242_gb300.lattice import Lattice
+from test_gpu_final_sums import us_a_call
+
+pytestmark = pytest.mark.gpu
+
+
+def _times(nx, ny, shape, steps):
+    with Lattice(nx, ny, 1 / 3, 0.6, "complete", "f32") as lat:
+        lat.init(*(torch.from_numpy(a).cuda() for a in flows.shear_wave(nx, ny, U=0.1, amp=0.01)))
+        default = us_a_call(lat, steps)
+        capi.lbm_set_launch_ex(lat.ctx, *shape)
+        return default, us_a_call(lat, steps)
+
+
+@pytest.mark.parametrize("nx,ny,rows", [(1200, 1200, 6), (1800, 1800, 12), (2000, 734, 6), (1470, 1122, 6), (3467, 1744, 24)])
+def test_two_steps_a_launch(nx, ny, rows):
+    default, other = _times(nx, ny, (2, 0, 1, rows), 20)
+    assert default < 1.03 * other
