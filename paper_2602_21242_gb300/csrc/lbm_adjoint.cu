@@ -380,7 +380,7 @@ cudaError_t fwd_step(lbm_ctx* c, const void* src, void* dst) {
   a.tau = c->tau;
   a.rho_ref = c->rho_ref;
   a.partials = c->d_parts;
-  a.cfg = c->cfg;
+  a.cfg = c->single_cfg();
   a.err = c->d_err;
   a.sched = c->d_sched;
   cudaError_t e = c->prec == LBM_F64      ? olbm::launch_step_f64(a, c->stream)

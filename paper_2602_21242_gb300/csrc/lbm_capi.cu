@@ -131,6 +131,20 @@ int diag_rows(const olbm::Geometry& g, olbm::LaunchCfg k, int prec, int sms) {
   return std::max(rows_for(17.0), std::min(5, rows_for(4.4)));
 }
 
+// Rows of the single steps under the default two-step launch of the FP32 form (calls of one step, the last of an
+// odd count, lattices with walls, states recomputed for the adjoint): their CTAs (kind 1) are three an SM
+// and strips of their own width, so the two-step launch's rows leave a part-filled second wave. One wave while
+// that takes at most 24 rows, else two or three of equal height; large lattices as the two-step launch. us a
+// call of one step, by the two-step launch's rows -> these: 700^2 9.5 -> 7.0, 1000^2 14.6 -> 11.1, 4096 x 300 18.2 ->
+// 13.1, 1200^2 20.5 -> 16.5, 2048^2 53.2 -> 48.5.
+int single_rows(const olbm::Geometry& g, const olbm::LaunchCfg& cfg, int prec, int sms) {
+  if (prec != LBM_F32_SHIFT || cfg.kind != 2) return 0;
+  const long long wave = (long long)olbm::stream_ctas_per_sm(prec) * sms;
+  const long long strips = (g.nx + olbm::stream_tile_width(prec) - 1) / olbm::stream_tile_width(prec);
+  const long long work = strips * g.ny, waves = (work + 24 * wave - 1) / (24 * wave);
+  return waves <= 3 ? (int)((work + waves * wave - 1) / (waves * wave)) : 0;
+}
+
 // Diagnosed steps of a group: as many as fit half a MiB, at most eight and at least two (a two-step
 // launch diagnoses two). Grouping saves a few microseconds a step, which counts where a step has few
 // blocks, while eight buffers of a large lattice would be memory (640 bytes a block in place of 160) and
@@ -264,12 +278,15 @@ int lbm_create_ex(int nx, int ny, double theta, double tau, int model, int prec,
   c->cfg = default_cfg(prec, c->g, sms);
   c->nparts = olbm::step_blocks(c->g, c->cfg, prec);
   if (prec == LBM_F64 || prec == LBM_F64_DF) c->diag_rows = diag_rows(c->g, c->cfg, prec, sms);
+  c->single_rows = single_rows(c->g, c->cfg, prec, sms);
+  c->nparts = std::max(c->nparts, olbm::step_blocks(c->g, c->single_cfg(), prec));
   // FP32 / FP16 lattices with an odd width below 32 columns update single nodes (kind 0),
   // whose last bits differ from the node pairs of the tiles: they keep single steps.
   if (c->cfg.kind != 0 || prec == LBM_F64 || prec == LBM_F64_DF || nx % 2 == 0)
     for (int w = 0; w < 2; ++w) c->tile[w] = olbm::tile_plan(c->g, prec, theta, tau, sms, w != 0);
   c->default_cfg = c->cfg;
   c->default_diag_rows = c->diag_rows;
+  c->default_single_rows = c->single_rows;
   for (int w = 0; w < 2; ++w) c->default_tile[w] = c->tile[w];
   // (a cut into tiles has at most two an SM)
   // (diagnosed steps take at least as many rows, so no more partials, unless one row is all there is)
@@ -558,7 +575,8 @@ int lbm_step(lbm_ctx* ctx, int n) {
     a.src = ctx->buf[ctx->cur];
     a.dst = ctx->buf[ctx->cur ^ 1];
     used = ctx->nparts;
-    a.cfg.rows = a.diag && ctx->diag_rows > 0 ? ctx->diag_rows : ctx->cfg.rows;
+    a.cfg = two ? ctx->cfg : ctx->single_cfg();
+    if (a.diag && ctx->diag_rows > 0) a.cfg.rows = ctx->diag_rows;
     if (a.cfg.rows != ctx->cfg.rows) used = olbm::step_blocks(ctx->g, a.cfg, ctx->prec);
     cudaError_t e = reserve((a.diag ? 1 : 0) + (a.diag2 ? 1 : 0));
     if (e != cudaSuccess) return cuda_fail(ctx, e, "lbm_step diagnostics launch");
@@ -780,6 +798,7 @@ int lbm_set_launch_ex(lbm_ctx* ctx, int kind, int bx, int by, int rows) {
   const bool dflt = olbm::same_shape(k, ctx->default_cfg);
   ctx->cfg = dflt ? ctx->default_cfg : k;
   ctx->diag_rows = dflt ? ctx->default_diag_rows : 0;
+  ctx->single_rows = dflt ? ctx->default_single_rows : 0;
   for (int w = 0; w < 2; ++w) ctx->tile[w] = dflt ? ctx->default_tile[w] : olbm::TilesPlan{};
   ctx->nparts = need;
   return LBM_OK;

@@ -19,14 +19,20 @@ struct lbm_ctx {
   bool initialised = false;
   cudaStream_t stream = nullptr;
   olbm::LaunchCfg cfg{};
-  int diag_rows = 0;  // rows of a diagnosed step under the default FP64 launch (0: as cfg)
+  int diag_rows = 0;    // rows of a diagnosed step under the default FP64 launch (0: as cfg)
+  int single_rows = 0;  // rows of the single steps under the default two-step launch (0: as cfg)
   // several steps a launch on small lattices, without and with walls; off while lbm_set_launch's shape is another
   // than the default one
   olbm::TilesPlan tile[2]{};
-  // the three as lbm_create chose them: lbm_set_launch of that shape brings them back
+  // all of them as lbm_create chose them: lbm_set_launch of that shape brings them back
   olbm::LaunchCfg default_cfg{};
-  int default_diag_rows = 0;
+  int default_diag_rows = 0, default_single_rows = 0;
   olbm::TilesPlan default_tile[2]{};
+  olbm::LaunchCfg single_cfg() const {  // of a step that is not diagnosed
+    olbm::LaunchCfg k = cfg;
+    if (single_rows > 0) k.rows = single_rows;
+    return k;
+  }
   // Per-block diagnostics partials: kGroups groups of group_jobs buffers of parts_cap
   // blocks each, in one allocation (its start also serves lbm_diagnostics). Diagnosed steps
   // fill a group's buffers in turn; the final sums of a group that is full, or that the last diagnosed

@@ -23,3 +23,9 @@ def _times(nx, ny, shape, steps):
 def test_two_steps_a_launch(nx, ny, rows):
     default, other = _times(nx, ny, (2, 0, 1, rows), 20)
     assert default < 1.03 * other
+
+
+@pytest.mark.parametrize("nx,ny,rows", [(650, 650, 3), (700, 700, 3), (1116, 424, 3), (900, 900, 6), (4096, 300, 6), (2048, 2048, 24)])
+def test_single_steps(nx, ny, rows):
+    default, other = _times(nx, ny, (1, 0, 1, rows), 1)
+    assert default < 1.03 * other
