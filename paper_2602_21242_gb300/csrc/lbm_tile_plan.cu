@@ -37,10 +37,13 @@ TilesPlan tile_plan(const Geometry& g, int prec, double theta, double tau, int s
   if (f64 && !fx::make_coefs(theta, tau).on) return best;  // the tiles take the fixed-point collision
   const Cost k = cost_of(prec);
   const int elem = prec == 1 ? 4 : (prec == 2 ? 2 : 8);
-  const double single = (f64 ? 2.2 : 2.3) + (double)g.nx * g.ny * k.per_node + (walls ? 2.0 : 0.0);
-  // (FP16's single steps run up to a fifth below the fit on wide lattices: 2042 x 106 3.6 against
-  // 4.1 in tiles with the margin of the other forms)
-  double least = (prec == 2 ? 0.85 : 0.95) * single;
+  double single = (f64 ? 2.2 : 2.3) + (double)g.nx * g.ny * k.per_node;
+  // FP16's single steps take one row a CTA on these lattices and at most 3.35 while those are one wave of the three
+  // resident an SM, whatever the nodes (us a step in tiles / single: 391 x 383 3.8 / 3.6, 378 x 413
+  // 3.8 / 3.3, 450^2 3.8 / 3.5, 2042 x 106 4.3 / 3.5, 400^2 3.25 / 3.4; 512^2, two waves, 3.95 / 4.6).
+  const long long strips = (g.nx + stream_tile_width(2) - 1) / stream_tile_width(2);
+  if (prec == 2 && strips * g.ny <= (long long)stream_ctas_per_sm(2) * sms) single = std::min(single, 3.35);
+  double least = (prec == 2 ? 0.85 : 0.95) * (single + (walls ? 2.0 : 0.0));
   if (1.25 / 8 + k.L + (double)g.nx * g.ny * k.c / sms > least) return best;  // no cut can be cheaper
   for (int a = 1; a <= std::min(g.nx, 2 * sms); ++a) {
     const int tx = (g.nx + a - 1) / a;

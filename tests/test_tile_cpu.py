@@ -25,6 +25,19 @@ def checker(tmp_path_factory):
     return exe
 
 
+def _run(checker, *args):
+    out = subprocess.run([checker, *map(str, args)], capture_output=True, text=True, check=True).stdout
+    return [int(v) for v in out.split()]  # widths, planned, largest region, wrong indices
+
+
+@pytest.mark.parametrize("nx,ny,planned", [(378, 413, 0), (391, 383, 0), (450, 450, 0), (2042, 106, 0), (256, 256, 1),
+                                           (512, 512, 1), (984, 105, 1), (5000, 31, 1), (284, 670, 1)])
+def test_fp16_line_to_single_steps(checker, nx, ny, planned):
+    """FP16 single steps that are one wave of CTAs are faster than tiles from about 150,000 nodes (measured: 3.3 to
+    3.6 us a step against 3.8 to 4.3); below, and where they take two waves, the tiles are."""
+    assert _run(checker, 2, 0, 152, ny, nx, nx, 1)[1] == planned
+
+
 @pytest.mark.parametrize("prec", [0, 1, 2, 3])
 @pytest.mark.parametrize("walls", [0, 1])
 @pytest.mark.parametrize("ny", [1, 2, 3, 4, 5, 7, 20, 100])
@@ -34,9 +47,7 @@ def test_rows_of_every_planned_region(checker, prec, walls, ny):
     for sms, lo, hi, stride in [(152, 1, 10_000 // ny, 37), (152, 10_000 // ny, 1_000_000 // ny, 4999 // ny * 2 + 1),
                                 (148, 10_000 // ny, 1_000_000 // ny, 9973 // ny * 2 + 1), (20, 1, 100_000 // ny, 997),
                                 (1, 1, 5000, 61)]:
-        out = subprocess.run([checker, *map(str, (prec, walls, sms, ny, max(lo, 1), hi, stride))], capture_output=True,
-                             text=True, check=True).stdout
-        widths, planned, largest, wrong = map(int, out.split())
-        assert wrong == 0, (sms, lo, hi, out)
+        widths, planned, largest, wrong = _run(checker, prec, walls, sms, ny, max(lo, 1), hi, stride)
+        assert wrong == 0, (sms, lo, hi, largest)
         plans += planned
     assert plans > 0

@@ -10,6 +10,11 @@
 
 #include "lbm_tile_plan.cu"
 
+// (lbm_reduce.cu's, which needs a device)
+namespace olbm {
+int stream_tile_width(int prec) { return prec == 1 ? 256 : 512; }
+int stream_ctas_per_sm(int) { return 3; }
+}  // namespace olbm
 using namespace olbm;
 
 int main(int, char** v) {
