@@ -52,14 +52,18 @@ TilesPlan tile_plan(const Geometry& g, int prec, double theta, double tau, int s
       const int ty = (g.ny + b - 1) / b;
       if ((g.ny + ty - 1) / ty != b) continue;
       const int m = (a * b + sms - 1) / sms;
+      // no number of steps makes this cut cheaper than the best so far
+      if (1.25 / kTileStepsMax + k.L + (double)m * ((double)tx * ty) * k.c > least) continue;
       double work = 0.0;  // of the steps so far, last first (the region grows towards the first)
       for (int s = 1; s <= kTileStepsMax; ++s) {
         const int grow = 2 * (s - 1);
         if ((a > 1 && tx + grow > g.nx) || (b > 1 && ty + grow > g.ny)) break;  // a tile would meet itself
         const long long n = tile_nodes(g, tx, ty, s);
         if (tile_smem(g, tx, ty, s, elem) * m > kTileSmemMax) break;
-        work += k.L + (double)m * (double)n * k.c;
+        const double step = k.L + (double)m * (double)n * k.c;
+        work += step;
         const double t = (1.25 + work) / s;
+        if (step > least && t > least) break;  // and every further step costs as much
         if (s >= 2 && t < least) least = t, best.tx = tx, best.ty = ty, best.steps = s;
       }
     }

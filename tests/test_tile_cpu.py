@@ -27,7 +27,7 @@ def checker(tmp_path_factory):
 
 def _run(checker, *args):
     out = subprocess.run([checker, *map(str, args)], capture_output=True, text=True, check=True).stdout
-    return [int(v) for v in out.split()]  # widths, planned, largest region, wrong indices
+    return [int(v) for v in out.split()]  # widths, planned, largest region, wrong indices, dear plans
 
 
 @pytest.mark.parametrize("nx,ny,planned", [(378, 413, 0), (391, 383, 0), (450, 450, 0), (2042, 106, 0), (256, 256, 1),
@@ -47,7 +47,7 @@ def test_rows_of_every_planned_region(checker, prec, walls, ny):
     for sms, lo, hi, stride in [(152, 1, 10_000 // ny, 37), (152, 10_000 // ny, 1_000_000 // ny, 4999 // ny * 2 + 1),
                                 (148, 10_000 // ny, 1_000_000 // ny, 9973 // ny * 2 + 1), (20, 1, 100_000 // ny, 997),
                                 (1, 1, 5000, 61)]:
-        widths, planned, largest, wrong = _run(checker, prec, walls, sms, ny, max(lo, 1), hi, stride)
-        assert wrong == 0, (sms, lo, hi, largest)
+        widths, planned, largest, wrong, dear = _run(checker, prec, walls, sms, ny, max(lo, 1), hi, stride)
+        assert wrong == 0 and dear == 0, (sms, lo, hi, largest)
         plans += planned
     assert plans > 0
