@@ -259,12 +259,13 @@ __device__ __forceinline__ double widen_hi(float f) {
   return __hiloint2double((int)hw, (int)(u << 29));
 }
 // The same widening with FP32 subnormals flushed to a signed zero (for the low
-// part, whose subnormal values must not widen to 2^-127).
+// part, whose subnormal values must not widen to 2^-127), and infinities and NaNs
+// kept (a rebiased exponent alone made a NaN 1.4e39, a finite population).
 __device__ __forceinline__ double widen_lo(float f) {
-  const unsigned u = __float_as_uint(f);
-  const unsigned neg = (unsigned)((int)u >> 31) & 0x70000000u;
-  const unsigned hw = (u & 0x7F800000u) == 0u ? (u & 0x80000000u) : (u >> 3) + 0x38000000u + neg;
-  return __hiloint2double((int)hw, (u & 0x7F800000u) == 0u ? 0 : (int)(u << 29));
+  const unsigned u = __float_as_uint(f), e = u & 0x7F800000u;
+  const unsigned neg = (unsigned)((int)u >> 31) & 0x70000000u, bias = e == 0x7F800000u ? 0x70000000u : 0x38000000u;
+  const unsigned hw = e == 0u ? (u & 0x80000000u) : (u >> 3) + bias + neg;
+  return __hiloint2double((int)hw, e == 0u ? 0 : (int)(u << 29));
 }
 __device__ __forceinline__ double join_f64(df64 v) { return widen_hi(v.hi) + (double)v.lo; }
 // Both parts widened with integer instructions: one FP64-pipe instruction a value.
