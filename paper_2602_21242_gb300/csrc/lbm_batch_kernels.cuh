@@ -72,6 +72,9 @@ __global__ void __launch_bounds__(512) batch_persistent_kernel(const Desc<typena
       const int4 tl = tiles[t];
       const Desc<typename Form<PREC>::T> d = desc[tl.x];
       update_tile<MODEL, PREC, false, true>(d, tl.y, tl.z, parity, rows, nullptr);
+      // Lanes beyond the domain's width are done at once. Without this they run ahead into tiles of other
+      // domains, with other row counts, while the rest of their warp votes.
+      __syncwarp();
     }
     if (!grid_sync(bar, gridDim.x)) return;
   }

@@ -389,12 +389,11 @@ template <int MODEL, int PREC, bool DIAG, bool PAIRS, bool CG = false> struct Co
                                                DiagAcc<CT>& acc, FixedDiagAcc& facc) {
     using Raw = Column<MODEL, 0, DIAG, false, CG>;
     int mode = 0;  // FP64: which products this warp's nodes take (see collide)
-    const unsigned warp = __activemask();
     double f[9];
     bool loaded = false;
     for (int r = 0, y = y0; r < rows && y < g.ny; ++r, y += dy) {
       const bool mine = (left >> r) & 1;
-      if (!__any_sync(warp, mine)) continue;
+      if (!__any_sync(__activemask(), mine)) continue;  // (a mask kept over the loop could hold lanes that left it)
       if (mine) {
         if (!loaded) Raw::pull(src, g, x, xm, xp, y, f);
         loaded = (r + 1 < rows) && (y + dy < g.ny) && ((left >> (r + 1)) & 1);
@@ -442,7 +441,6 @@ template <int MODEL, int PREC, bool DIAG, bool PAIRS, bool CG = false> struct Co
           for (int i = 0; i < 9; ++i) f[i] = fn[i];
         }
       }
-      __syncwarp(warp);
     }
   }
 
