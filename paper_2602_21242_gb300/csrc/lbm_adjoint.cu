@@ -157,7 +157,7 @@ template <int MODEL>
 __global__ void __launch_bounds__(kAFX* kAFY, OLBM_ADJ_F64_MINB) adj_step_f64_kernel(const double* fbuf,
                                                                                      const double* lam_next, double* lam,
                                                                                      Geometry g, Coef<double> c) {
-  const int x = blockIdx.x * kAFX + threadIdx.x, y = blockIdx.y * kAFY + threadIdx.y;
+  const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y;
   pdl_wait();
   pdl_launch_dependents();
   if (x >= g.nx || y >= g.ny) return;
@@ -300,8 +300,11 @@ template <int PREC> struct Adjoint {
       }
     }
     if constexpr (PREC == 0) {
-      const dim3 grid((g.nx + kAFX - 1) / kAFX, (g.ny + kAFY - 1) / kAFY);
-      return launch_step_kernel(adj_step_f64_kernel<MODEL>, grid, dim3(kAFX, kAFY), 0, st, (const double*)fbuf,
+      // two rows a block, or kABY where the grid would have more than 65535 rows of them (ny > 131070)
+      const bool tall = (g.ny + kAFY - 1) / kAFY > 65535;
+      const dim3 block = tall ? dim3(kAFX * kAFY / kABY, kABY) : dim3(kAFX, kAFY);
+      const dim3 grid((g.nx + block.x - 1) / block.x, (g.ny + block.y - 1) / block.y);
+      return launch_step_kernel(adj_step_f64_kernel<MODEL>, grid, block, 0, st, (const double*)fbuf,
                                 (const double*)lam_next, (double*)lam, g, c);
     } else {
       adj_step_kernel<MODEL, PREC><<<adj_grid(g), dim3(kABX, kABY), 0, st>>>((const S*)fbuf, (const T*)lam_next,
