@@ -62,17 +62,30 @@ enum lbm_model {
 };
 
 /* Storage / arithmetic forms.
- *   LBM_F64        populations stored in FP64, all arithmetic in FP64.
+ *   LBM_F64        populations stored in FP64. A node whose populations are below 1
+ *                  in magnitude, density in [1/2, 4), velocity components below
+ *                  1/2 and normal and shear non-equilibrium stresses below 1/2,
+ *                  with theta in [0.21, 0.65] and tau at most 1e9, collides in
+ *                  64-bit fixed point: populations are taken exactly down to 2^-8
+ *                  and truncated at 2^-60 below, sums are exact, products are
+ *                  kept to 2^-60 and the result is rounded to binary64 once.
+ *                  Every other node collides in FP64 arithmetic (several times
+ *                  slower, as is a flow in another unit of density). The
+ *                  choice depends on the node alone. lbm_init, lbm_moments and
+ *                  lbm_diagnostics take the same range of densities in fixed
+ *                  point and the rest in FP64.
  *   LBM_F32_SHIFT  stored as deviations f_i - rho_ref w_i(theta) in FP32, where
  *                  w_i(theta) is the rest GEq (Eq. 10 at u = 0) and rho_ref = 1;
  *                  collision arithmetic in FP32, reductions in FP64.
  *   LBM_F16_SHIFT  as LBM_F32_SHIFT with the deviations stored in IEEE FP16.
- *   LBM_F64_DF     populations stored in FP64 (the LBM_F64 layout), collision
- *                  arithmetic in double-float: each value the unevaluated sum of
+ *   LBM_F64_DF     populations stored in FP64 (the LBM_F64 layout), collision as
+ *                  LBM_F64 for nodes in the fixed-point range and
+ *                  in double-float for the others: each value the unevaluated sum of
  *                  two FP32 numbers (about 48 significant bits, FP32 exponent
  *                  range; magnitudes below 1.2e-38 become zero), built from
  *                  error-free transformations on the FP32 pipes. Same results
- *                  as LBM_F64 to about 1e-13 relative per step. Step launches
+ *                  as LBM_F64, for nodes outside the range to about 1e-13
+ *                  relative per step. Step launches
  *                  of at most 256 threads a block; lbm_vjp runs its adjoint in
  *                  double-float too; not available to the batched form. */
 enum lbm_prec {
@@ -152,10 +165,13 @@ int lbm_init(lbm_ctx* ctx, const double* d_rho, const double* d_ux, const double
  * Asynchronous. If a diagnostics interval M > 0 is set, every step whose start
  * time t is a multiple of M also reduces the diagnostics of f(x, t) (see
  * lbm_diagnostics) on the device; lbm_sync / lbm_step_diagnostics report them.
- * The final sums of those reductions run on a second stream that the context
- * owns, beside the following steps; before returning, the call makes the
+ * The final sums of those reductions run in groups of up to eight steps on a
+ * second stream that the context owns, beside the following steps (those of a
+ * call's last steps on its own stream); before returning, the call makes the
  * context's stream wait for them, so work queued on that stream afterwards sees
- * every result of the call.
+ * every result of the call. Small lattices (up to about 150^2 nodes in FP64
+ * storage, 600^2 in FP32, between 400^2 and 550^2 in FP16; more with walls) run several
+ * steps a launch, bit-identical to single steps, between diagnosed steps.
  * Errors: LBM_ESTATE before lbm_init or lbm_set_state; LBM_EINVAL for n < 0.
  */
 int lbm_step(lbm_ctx* ctx, int n);
@@ -340,9 +356,11 @@ int lbm_get_launch(const lbm_ctx* ctx, int* bx, int* by, int* rows);
  * LBM_ETIMEOUT. Same results as kind 0 for even nx (FP32 rounding may differ in
  * the last bit for odd nx, where kind 0 updates single nodes) except the
  * diagnostics' summation order. Default for the shifted forms on lattices at
- * least 32 columns wide: FP32 kind 2 below on 24-row tiles (48 from 8192^2); FP16 one CTA
+ * least 32 columns wide: FP32 kind 2 below on 24-row tiles (48 from 8192^2; smaller
+ * lattices the rows that make one or two whole waves of CTAs); FP16 one CTA
  * per tile with the height in {48, 40, 32, 24, 16} that best fills the last
- * wave of CTAs (halved further on small lattices).
+ * wave of CTAs (halved further on small lattices). FP64 storage: kind 0 with 64 x 2
+ * threads and up to 32 rows, fewer on smaller lattices (at least 20 CTAs an SM).
  * kind 2 (shifted FP32/FP16 forms; bx = 0, by ignored): two steps per launch
  * (temporal blocking of Eq. 1): each CTA computes step t's post-collision values
  * on its tile of 254 (FP32) or 510 (FP16) columns by `rows` rows plus a
@@ -351,7 +369,8 @@ int lbm_get_launch(const lbm_ctx* ctx, int* bx, int* by, int* rows);
  * two steps. Results are bit-identical to two single steps (the diagnostics'
  * summation order aside). It applies where two steps of a call follow each
  * other and no walls are set (any nx); other steps (the last of an odd
- * count) take kind 1 with one CTA per tile of the same height.
+ * count) take kind 1 with one CTA per tile of the same height (FP32's default: of
+ * the height that makes whole waves of those CTAs).
  */
 int lbm_set_launch_ex(lbm_ctx* ctx, int kind, int bx, int by, int rows);
 int lbm_get_launch_ex(const lbm_ctx* ctx, int* kind, int* bx, int* by, int* rows);
@@ -409,7 +428,7 @@ int lbm_batch_get_launch(const lbm_batch* b, int* bx, int* by, int* rows, int* n
  * 64, 128 or 256 (FP16), 0 = 128 (FP32) / 256 (FP16); narrower tiles waste less
  * of a strip on narrow domains. by is ignored. A domain's results equal those of
  * a single lattice stepped with the same launch kind. kind 2 (shifted forms, bx =
- * 0; the FP32 default, 32 rows): two steps a launch (the two-step tile routine
+ * 0; the FP32 default, up to 32 rows): two steps a launch (the two-step tile routine
  * of the single-lattice kind 2 on tiles of 254 (FP32) or 510 (FP16) columns x
  * rows rows of every domain, any width): in graph mode n / 2 two-step launches,
  * in persistent mode one cooperative launch looping over n / 2 pairs of steps;

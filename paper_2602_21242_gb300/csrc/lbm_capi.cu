@@ -59,11 +59,11 @@ long long nodes_of(const lbm_ctx* c) { return (long long)c->nx * c->ny; }
 // FP64 storage the column kernel with 64 x 2 threads and up to 32 rows per thread, fewer
 // on smaller lattices so that the grid has at least 20 CTAs per SM (four waves of the five
 // resident: 2048^2 6 to 10 rows 125-126 us a step, 32 rows 136; 1531 x 1277 2 to 6 rows
-// 61.6, 16 rows 69.6; diagnosed steps take more rows, see diag_rows); the shifted forms the bulk-copy pipeline with one CTA per tile of 32
-// rows (refined per form below), except on lattices narrower than 32 columns, where the
-// column kernel with 128 x 4 threads and 16 rows wastes fewer threads. On smaller lattices
-// their rows are halved until the grid has at least 4 CTAs per SM.
-// lbm_set_launch[_ex] (and the autotuner built on it) overrides the choice.
+// 61.6, 16 rows 69.6; diagnosed steps take more rows, see diag_rows); the shifted forms the
+// bulk-copy pipeline with one CTA per tile of 32 rows (refined per form below), except on
+// lattices narrower than 32 columns, where the column kernel with 128 x 4 threads and 16 rows
+// wastes fewer threads. On smaller lattices their rows are halved until the grid has at least
+// 4 CTAs per SM. lbm_set_launch[_ex] (and the autotuner built on it) overrides the choice.
 olbm::LaunchCfg default_cfg(int prec, const olbm::Geometry& g, int sms) {
   olbm::LaunchCfg k;
   if (prec == LBM_F64 || prec == LBM_F64_DF) {

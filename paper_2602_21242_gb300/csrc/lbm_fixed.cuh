@@ -49,7 +49,7 @@
 // alone: 7), and 1000 steps of a decaying Taylor-Green vortex drift in mass by 7e-17
 // (binary64: 1.1e-13, from the rounding of 1 - theta).
 //
-// Measured (GB300, 4096^2, complete model, diagnostics every step): 6.33 -> 31.8 GLUPS.
+// Measured (GB300, 4096^2, complete model, diagnostics every step): 6.33 -> 34.0 GLUPS.
 //
 // The routines compile for the host as well, where tests compare them with
 // extended-precision arithmetic.

@@ -612,7 +612,7 @@ __global__ void __launch_bounds__(512) step_kernel(const typename Form<PREC>::S*
 // form's, double-word arithmetic for the nodes outside its range and for temperatures it
 // does not take. Launched with at most 256 threads a block and capped at 96 registers a
 // thread, five blocks of 128 threads per SM. The complete model with fused diagnostics at
-// 4096^2: 30.8 GLUPS (25.2 with every node in double-word arithmetic; that with 80 and 88
+// 4096^2: 33.4 GLUPS (25.2 with every node in double-word arithmetic; that with 80 and 88
 // registers 24.7 and 25.0).
 #ifndef OLBM_DF_MAXNREG
 #define OLBM_DF_MAXNREG 96
@@ -625,11 +625,12 @@ __global__ void __maxnreg__(OLBM_DF_MAXNREG) step_kernel_df(const double* src, d
 }
 
 // The FP64 form collides in 64-bit fixed point on the integer pipes (lbm_fixed.cuh),
-// which bound it: ALU, FMA-heavy (the wide products) and issue are each about 60 %
-// busy. Complete model at 4096^2, diagnostics every step / off: 31.8 / 34.5 GLUPS
+// which bound it: ALU 64 % busy, the wide products beside it, no pipe full. Complete
+// model at 4096^2, diagnostics every step / off: 34.0 / 35.3 GLUPS
 // (6.33 / 6.8 with the collision on the FP64 pipe, its products on the integer pipes).
 // Capped at 96 registers a thread, five blocks of 128 threads an SM, without spills in
-// the row loop (128: 31.6 / 33.2, 88: 31.7 / 34.0, 80: 32.1 / 34.1, 72: 31.6 / 33.7).
+// the row loop (before 32-bit offsets, 96: 31.8 / 34.5, 128: 31.6 / 33.2, 88: 31.7 / 34.0, 80:
+// 32.1 / 34.1, 72: 31.6 / 33.7).
 // Launched with at most 512 threads.
 #ifndef OLBM_F64_MAXNREG
 #define OLBM_F64_MAXNREG 96

@@ -12,8 +12,8 @@
 //   and 10.0 at 64^2, 256^2, 384^2 and 512^2) or 2.3 + nodes / 100e3 (FP32, FP16: 2.4,
 //   3.2, 4.8 and 12.2 at 64^2, 256^2, 512^2 and 1024^2).
 // So the line lies near 150^2 nodes for FP64 storage (64^2: 2.45 -> 1.9 us a step, 256^2
-// stays at 4.5 against 4.8 in tiles) and near 600^2 for FP32 and FP16 (512^2 4.8 -> 3.8,
-// 768^2 7.6 against 8.3). Walls cost the single steps another launch (about 2 us), which the
+// stays at 4.5 against 4.8 in tiles) and near 600^2 for FP32 (512^2 4.8 -> 3.8,
+// 768^2 7.6 against 8.3); for FP16 between 390^2 and 550^2, by the waves of its single steps. Walls cost the single steps another launch (about 2 us), which the
 // tiles do not need, so lattices with walls take tiles up to a higher line.
 #include "lbm_tile.h"
 

@@ -72,7 +72,8 @@ def _key(kind: str, nodes: int, prec: int, model: int, extra: str = "") -> str:
 def _timing_fields(nx: int, ny: int):
     """(rho, ux, uy) host arrays the candidates are timed on: the advected shear wave of the
     bandwidth benchmark (u_x = 0.1, u_y = 0.01 sin(2 pi x / nx)). A fluid at rest would time
-    another code path of the FP64 form, whose products take zero operands on a slower path."""
+    another code path of the FP64 form at temperatures outside its fixed-point range, where
+    products take zero operands on a slower path."""
     return flows.shear_wave(nx, ny, U=0.1, amp=0.01)
 
 
