@@ -447,7 +447,7 @@ template <int MODEL, int PREC, bool DIAG, bool PAIRS, bool CG = false> struct Co
   // FP64 storage: the rows of a column in fixed point; returns the rows it left out, which are
   // all rows from the first one on that has no node of the warp in range. (In a flow of another unit of
   // density, or faster than 1/2, that is the first: us a step at 4096^2, density 10, with every row tried first -> now,
-  // and with every node in the form's own arithmetic inline: FP64 2751 -> 2714, 2474; double-word 889 -> 787,
+  // and with every node in the form's own arithmetic inline: FP64 2751 -> 2700, 2474; double-word 889 -> 777,
   // 624. Those rows inline here as well would take that to 2518 and 657, but slow the rows in range down by
   // 2 to 3 % through their registers.) Byte
   // offsets inside a plane as OFF: 32 bits where a plane is below 4 GiB, so that the nine

@@ -13,7 +13,7 @@ from paper_2602_21242_gb300.lattice import Lattice
 pytestmark = pytest.mark.gpu
 
 
-def us_a_call(lat, steps, calls=20, reps=9):
+def us_a_call(lat, steps, calls=20, reps=15):
     best = float("inf")
     for _ in range(reps):
         e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
